@@ -105,14 +105,7 @@ __global__ void __launch_bounds__(256) k_heights(const HeightsLaunch a) {
   const long long excl = block_scan_incl(tot, warp_tot) - tot;
   long long h = excl, s1 = 0;
   unsigned long long s2 = 0;
-  for (uint32_t i = w0; i < w1; ++i) {
-    const uint32_t x = w[i];
-    for (uint32_t b = 0; b < 32; ++b) {
-      h += ((x >> b) & 1u) ? 1 : -1;
-      s1 += h;
-      s2 += static_cast<unsigned long long>(h * h);
-    }
-  }
+  for (uint32_t i = w0; i < w1; ++i) add_word_heights(w[i], h, s1, s2);
   const long long s1_all = block_scan_incl(s1, warp_tot);  // last thread holds the total
   // sum of h^2 can exceed 2^64 for L = 2^22: warp sums (< 2^63) then 128 bits
 #pragma unroll
@@ -168,14 +161,7 @@ __global__ void __launch_bounds__(256) k_heights_part(const HeightsLaunch a, uin
   const long long incl = block_scan_incl(tot, warp_tot);
   long long h = incl - tot, s1 = 0;
   unsigned long long s2 = 0;
-  for (uint32_t i = w0; i < w1; ++i) {
-    const uint32_t x = w[i];
-    for (uint32_t b = 0; b < 32; ++b) {
-      h += ((x >> b) & 1u) ? 1 : -1;
-      s1 += h;
-      s2 += static_cast<unsigned long long>(h * h);
-    }
-  }
+  for (uint32_t i = w0; i < w1; ++i) add_word_heights(w[i], h, s1, s2);
   const long long s1_all = block_scan_incl(s1, warp_tot);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
@@ -370,14 +356,7 @@ __device__ void record_heights_cl(const cg::cluster_group& cl, uint32_t* cur, co
     long long s1 = 0;
     unsigned long long s2 = 0;
     if (ln.active) {
-      for (uint32_t r = 0; r < a.R2; ++r) {
-        const uint32_t x = pl[r * a.Cp + ln.c];
-        for (uint32_t b = 0; b < 32; ++b) {
-          h += ((x >> b) & 1u) ? 1 : -1;
-          s1 += h;
-          s2 += static_cast<unsigned long long>(h * h);
-        }
-      }
+      for (uint32_t r = 0; r < a.R2; ++r) add_word_heights(pl[r * a.Cp + ln.c], h, s1, s2);
     }
     const long long t1 = block_scan_incl(s1, warp_tot);
     const long long t2 = block_scan_incl(static_cast<long long>(s2), warp_tot);  // slice sum < 2^62

@@ -127,21 +127,15 @@ __device__ void record_heights(const uint32_t* cur, const DomainLaunch& a, uint3
       for (uint32_t r = 0; r < a.R2; ++r) tot += 2 * __popc(pl[r * a.Cp + ln.c]) - 32;
     long long h0, seg_unused;
     seg_scan(tot, ln.col0, a.G, warp_tot, arr, h0, seg_unused);
-    long long s1 = 0, s2 = 0;
+    long long s1 = 0;
+    unsigned long long s2 = 0;
     if (ln.active) {
       long long h = h0;
-      for (uint32_t r = 0; r < a.R2; ++r) {
-        const uint32_t x = pl[r * a.Cp + ln.c];
-        for (uint32_t b = 0; b < 32; ++b) {
-          h += ((x >> b) & 1u) ? 1 : -1;
-          s1 += h;
-          s2 += h * h;
-        }
-      }
+      for (uint32_t r = 0; r < a.R2; ++r) add_word_heights(pl[r * a.Cp + ln.c], h, s1, s2);
     }
     long long e1, t1, e2, t2;
     seg_scan(s1, ln.col0, a.G, warp_tot, arr, e1, t1);
-    seg_scan(s2, ln.col0, a.G, warp_tot, arr, e2, t2);
+    seg_scan(static_cast<long long>(s2), ln.col0, a.G, warp_tot, arr, e2, t2);
     if (ln.active && ln.g == 0) {
       const size_t e = (static_cast<size_t>(slot) * a.geo.S + ln.sample) * NOCC + p;
       a.tab_sh[e] = t1;

@@ -423,14 +423,7 @@ __device__ void sca_record(const uint32_t* lat, const DomainLaunch& a, uint32_t 
     for (uint32_t i = w0; i < w1; ++i) tot += 2 * __popc(pl[i]) - 32;
     long long h = block_scan_incl(tot, warp_tot) - tot, s1 = 0;
     unsigned long long s2 = 0;
-    for (uint32_t i = w0; i < w1; ++i) {
-      const uint32_t x = pl[i];
-      for (uint32_t b = 0; b < 32; ++b) {
-        h += ((x >> b) & 1u) ? 1 : -1;
-        s1 += h;
-        s2 += static_cast<unsigned long long>(h * h);
-      }
-    }
+    for (uint32_t i = w0; i < w1; ++i) add_word_heights(pl[i], h, s1, s2);
     const long long s1_all = block_sum(s1, warp_tot);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);

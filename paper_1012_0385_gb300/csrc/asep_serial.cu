@@ -168,14 +168,7 @@ __global__ void __launch_bounds__(256) k_serial(const SerialLaunch a) {
         h -= tot;
         long long s1 = 0;
         unsigned long long s2 = 0;
-        for (uint32_t w = w0; w < w1; ++w) {
-          const uint32_t xw = pw[w];
-          for (uint32_t bb = 0; bb < 32; ++bb) {
-            h += ((xw >> bb) & 1u) ? 1 : -1;
-            s1 += h;
-            s2 += static_cast<unsigned long long>(h * h);
-          }
-        }
+        for (uint32_t w = w0; w < w1; ++w) add_word_heights(pw[w], h, s1, s2);
         // profile and autocorrelation overlap of this plane
         const size_t pbase = (static_cast<size_t>(sample) * NOCC + p) * W;
         long long ov = 0;
@@ -418,14 +411,7 @@ __global__ void __launch_bounds__(1024) k_serial_rounds(const SerialLaunch a) {
         long long h = block_scan_incl(tot, s_i64) - tot;
         long long s1 = 0;
         unsigned long long s2 = 0;
-        for (uint32_t w = w0; w < w1; ++w) {
-          const uint32_t xw = pw[w];
-          for (uint32_t bb = 0; bb < 32; ++bb) {
-            h += ((xw >> bb) & 1u) ? 1 : -1;
-            s1 += h;
-            s2 += static_cast<unsigned long long>(h * h);
-          }
-        }
+        for (uint32_t w = w0; w < w1; ++w) add_word_heights(pw[w], h, s1, s2);
         const size_t pbase = (static_cast<size_t>(sample) * NOCC + p) * W;
         long long ov = 0;
         for (uint32_t w = w0; w < w1; ++w) {
