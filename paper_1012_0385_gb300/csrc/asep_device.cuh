@@ -48,6 +48,54 @@ __device__ __forceinline__ uint4 philox10(uint4 c, const KeySchedule& ks) {
   return c;
 }
 
+// Philox4x32-10 split by what varies.  A warp's calls at one sweep differ only
+// in counter word 3 (domain, unit or site group) and in the call field of
+// word 1, so the first three rounds need not be run per lane and call:
+//   round 1: both products (of words 0 and 2) are the same for all lanes;
+//   round 2: its product of word 0 depends on the call only, that of word 2
+//            on word 3 only;
+//   round 3: the same, the other way round.
+// A call then costs a lane 7 rounds (14 wide multiplies, the unit a plain
+// call saturates at 30.2 of 32 a clock and SM) and two XORs instead of 10
+// rounds; the per-call part (PhiloxHead) is formed once per sweep and sample,
+// the per-lane part (PhiloxLane) once per sweep, lane and counter word 3.
+struct PhiloxHead {
+  uint32_t c3, y3, d3;  // round 3 of one (sweep, call, sample): x ^= c3, word y, z ^= d3
+};
+struct PhiloxLane {
+  uint32_t y2, hv, w3;  // rounds 2 and 3 of one (sweep, sample, word 3)
+};
+
+// Round 1 of counter word 0: hi(M0 x) ^ ky0, to be XORed with counter word 3.
+__device__ __forceinline__ uint32_t philox_a0(uint32_t x, const KeySchedule& ks) {
+  return mul_wide(0xD2511F53u, x).y ^ ks.y[0];
+}
+
+__device__ __forceinline__ PhiloxHead philox_head(uint32_t x, uint32_t y, uint32_t z, const KeySchedule& ks) {
+  const uint2 q = mul_wide(0xD2511F53u, mul_wide(0xCD9E8D57u, z).y ^ y ^ ks.x[0]);  // round 2, word 0
+  const uint2 r = mul_wide(0xCD9E8D57u, q.y ^ mul_wide(0xD2511F53u, x).x ^ ks.y[1]);  // round 3, word 2
+  return {r.y ^ ks.x[2], r.x, q.x ^ ks.y[2]};
+}
+
+// b2 = philox_b2(z): round 2's XOR of counter word 2's low product.
+__device__ __forceinline__ uint32_t philox_b2(uint32_t z, const KeySchedule& ks) {
+  return mul_wide(0xCD9E8D57u, z).x ^ ks.x[1];
+}
+
+__device__ __forceinline__ PhiloxLane philox_lane(uint32_t a0, uint32_t b2, uint32_t w) {
+  const uint2 t = mul_wide(0xCD9E8D57u, a0 ^ w);
+  const uint2 v = mul_wide(0xD2511F53u, t.y ^ b2);
+  return {t.x, v.y, v.x};
+}
+
+// Rounds 4 to 10: = philox10 of the counter the head and the lane part came from.
+__device__ __forceinline__ uint4 philox_tail(const PhiloxHead& h, const PhiloxLane& l, const KeySchedule& ks) {
+  uint4 c = make_uint4(h.c3 ^ l.y2, h.y3, l.hv ^ h.d3, l.w3);
+#pragma unroll
+  for (int round = 3; round < 10; ++round) c = philox_round(c, ks.x[round], ks.y[round]);
+  return c;
+}
+
 __device__ __forceinline__ uint2 key_of(uint64_t seed) {
   return make_uint2(static_cast<uint32_t>(seed), static_cast<uint32_t>(seed >> 32));
 }

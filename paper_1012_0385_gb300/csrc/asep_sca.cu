@@ -28,12 +28,10 @@
 
 #include "asep_device.cuh"
 #include "asep_internal.h"
+#include "asep_sca.cuh"
 
 namespace asep {
 namespace {
-
-constexpr uint32_t kEven = 0x55555555u;
-constexpr uint32_t kOdd = 0xAAAAAAAAu;
 
 // Sum of per-thread values over the block; every thread gets the total.
 __device__ long long block_sum(long long v, long long* warp_tot) {
@@ -45,15 +43,6 @@ __device__ long long block_sum(long long v, long long* warp_tot) {
   __syncthreads();
   return t;
 }
-
-// Eight consecutive words (16-byte aligned) into registers.
-__device__ __forceinline__ void load8(const uint32_t* p, uint32_t (&x)[8]) {
-  const uint4 v0 = reinterpret_cast<const uint4*>(p)[0], v1 = reinterpret_cast<const uint4*>(p)[1];
-  x[0] = v0.x; x[1] = v0.y; x[2] = v0.z; x[3] = v0.w; x[4] = v1.x; x[5] = v1.y; x[6] = v1.z; x[7] = v1.w;
-}
-
-// All-ones where bit k (0 = most significant of 20) of a 20-bit threshold is set.
-__device__ __forceinline__ uint32_t bit_mask(uint32_t t20, uint32_t k) { return 0u - ((t20 >> (19u - k)) & 1u); }
 
 // Applies the accepted moves h[g] of a unit's four groups (bit 2j: bond j
 // of word 2g, bit 2j + 1: bond j of word 2g + 1) to its words; returns the
@@ -473,6 +462,221 @@ __device__ void sca_record(const uint32_t* lat, const DomainLaunch& a, uint32_t 
   __syncthreads();
 }
 
+// ---------------------------------------------------------------------------
+// One ring (or pair of lanes) per CTA, a unit per thread, in registers
+// ---------------------------------------------------------------------------
+
+// A thread keeps its unit's words in bond lanes (asep_sca.cuh) for the whole
+// launch; shared memory carries only what crosses a warp's ends (the next
+// unit's first site before the odd phase, the flip of it after), the shared
+// heads of the random calls, and the lattice at records.  Two barriers a
+// sweep, each behind the random planes of the following phase, which do not
+// depend on the lattice.  Threads beyond the ring's units run along on empty
+// words that nothing reads.
+// Bound by the integer ALU pipe (logic of Philox and of the update).  Measured
+// against units in shared memory as plain words (k_sca_smem), us per sweep:
+// 256 rings of 2^17 sites at p = 0.75, q = 0.25 3.17 -> 2.08, 128 pairs of
+// lanes of 2^16 with turning sites 11.0 -> 6.24, 201 rings of 391 units with
+// independent classes 18.8 -> 17.2 (its random planes dominate).
+template <uint32_t MODEL, bool DIS, bool COUNT, uint32_t FAST, bool PQ = false>
+__global__ void __launch_bounds__(DIS ? 512 : 1024) k_sca(const DomainLaunch a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ long long warp_tot[32];
+  __shared__ unsigned long long warp_s2[32];
+  __shared__ __align__(16) ScaHeads heads;
+  __shared__ uint32_t edge_e[2][32], edge_c[2][32];  // [lane][warp]: first unit's e[0]; flip into the next warp
+  constexpr uint32_t NOCC = MODEL == kTwoLane ? 2u : 1u;
+  constexpr int NQ = DIS ? (PQ ? 2 : 1) : 0;
+  constexpr bool TURNS = MODEL == kTwoLane && DIS;
+  const uint32_t W = a.geo.W, n_units = W / 8;
+  const uint32_t sample = blockIdx.x, n_glob = a.geo.first_sample + sample;
+  const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const uint32_t u = threadIdx.x;  // this thread's unit
+  const bool active = u < n_units;
+  const bool last = u + 1 == n_units || (lane == 31u && active);  // its next unit is another warp's first
+  const uint32_t wid_next = wid + 1 == nw ? 0u : wid + 1, wid_prev = (wid == 0 ? nw : wid) - 1;
+  uint32_t* lat = reinterpret_cast<uint32_t*>(smem_raw);  // NOCC planes of W words, for records
+  ScaTurnScratch* turn = reinterpret_cast<ScaTurnScratch*>(lat + NOCC * W);  // [nw] (turning sites)
+  const uint64_t s0 = a.clock->sweep;
+  uint32_t rec = a.clock->next_time;
+  const uint32_t kmax = a.sca_kmax, calls = sca_calls(kmax, TURNS), chunk = sca_chunk(calls);
+  const uint32_t b2 = philox_b2(n_glob, a.ks);
+
+  ScaUnit U[NOCC];
+  ScaUnit Q[NQ == 2 ? 2 : 1];  // ring: p (and q) classes; two lanes: turning sites, or the u and v marks
+  uint32_t q_odd[4] = {0u, 0u, 0u, 0u};  // ring: classes of the second sites of odd bonds
+  uint32_t* state = a.state + static_cast<size_t>(sample) * NOCC * W;
+#pragma unroll
+  for (uint32_t p = 0; p < NOCC; ++p) {
+    uint32_t x[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    if (active) load8(state + p * W + 8u * u, x);
+    U[p] = to_lanes(x);
+  }
+  if (DIS) {
+    const uint32_t* mask = a.mask + static_cast<size_t>(sample / a.geo.samples_per_real) * NQ * W;
+#pragma unroll
+    for (int p = 0; p < NQ; ++p) {
+      uint32_t x[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+      if (active) load8(mask + p * W + 8u * u, x);
+      Q[p] = to_lanes(x);
+    }
+    if (MODEL == kRing) {
+      constexpr int kq = NQ == 2 ? 1 : 0;
+      const uint32_t nx = active ? mask[kq * W + (u + 1 == n_units ? 0u : 8u * u + 8u)] : 0u;
+#pragma unroll
+      for (int g = 0; g < 4; ++g) q_odd[g] = odd_sites(Q[kq].e[g], g < 3 ? Q[kq].e[g + 1] : nx);
+    }
+  }
+  if (TURNS && !PQ) {
+    const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+    store8(turn[wid].flip[lane], zero);
+  }
+  if (lane == 0u) {
+    edge_c[0][wid] = 0u;
+    edge_c[1][wid] = 0u;
+  }
+
+  // The odd phase's flips into the first unit of a warp, left by the previous
+  // warp's last thread: taken at the next barrier, and cleared by whoever
+  // settles outside the loop.
+  auto settle = [&]() {
+    __syncthreads();
+    if (lane == 0u) {
+#pragma unroll
+      for (uint32_t p = 0; p < NOCC; ++p) U[p].e[0] ^= edge_c[p][wid_prev];
+    }
+  };
+  auto clear_edges = [&]() {
+    __syncthreads();
+    if (lane == 0u) {
+      edge_c[0][wid] = 0u;
+      edge_c[1][wid] = 0u;
+    }
+  };
+
+  ScaCounts cnt;
+  uint32_t filled = 0;  // sweeps of the launch whose heads have been formed
+  uint32_t base = 0;    // first of them in the current chunk
+  for (uint32_t it = 0; it < a.n_sweeps;) {
+    if (it == filled) {
+      __syncthreads();  // every warp is done with the previous chunk
+      base = it;
+      filled = min(it + chunk, a.n_sweeps);
+      sca_fill_heads(heads, s0 + it, filled - it, kmax, calls, n_glob, a.ks);
+      __syncthreads();
+    }
+    uint32_t stop = filled;  // next chunk or record
+    if (rec < a.n_times && a.times[rec] - s0 < stop) stop = static_cast<uint32_t>(a.times[rec] - s0);
+#pragma unroll 1
+    for (; it < stop; ++it) {
+      const uint4* hd = heads.head + (it - base) * calls;
+      const uint32_t a0 = heads.a0[it - base];
+      uint32_t h[4];
+      PhiloxLane pl[NOCC];
+      uint4 y0[NOCC], y1[NOCC];
+      // even phase; its planes come before the barrier
+#pragma unroll
+      for (uint32_t p = 0; p < NOCC; ++p) {
+        pl[p] = philox_lane(a0, b2, (2u * u) | (p << 31));
+        sca_first_planes<MODEL, FAST>(hd, pl[p], a.ks, y0[p], y1[p]);
+      }
+      if (!TURNS) settle();
+      sca_decide<MODEL, DIS, PQ, COUNT, FAST, 0, 0>(U[0], 0u, Q, q_odd, a.rates, kmax, hd, pl[0], y0[0], y1[0], a.ks,
+                                                    cnt, h);
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        U[0].e[g] ^= h[g];
+        U[0].o[g] ^= h[g];
+      }
+      if (MODEL == kTwoLane) {
+        sca_decide<MODEL, DIS, PQ, COUNT, FAST, 0, 1>(U[NOCC - 1], 0u, Q, q_odd, a.rates, kmax, hd, pl[NOCC - 1],
+                                                      y0[NOCC - 1], y1[NOCC - 1], a.ks, cnt, h);
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          U[NOCC - 1].e[g] ^= h[g];
+          U[NOCC - 1].o[g] ^= h[g];
+        }
+      }
+      if (TURNS)
+        cnt.c[2] += PQ ? sca_turn_all<0>(U[0], U[NOCC - 1], Q[0], u, active, a0, b2, hd[kmax], a)
+                       : sca_turn_pool<0>(U[0], U[NOCC - 1], Q[0], turn[wid], u, active, a0, b2, hd[kmax], a);
+      if (lane == 0u) {
+#pragma unroll
+        for (uint32_t p = 0; p < NOCC; ++p) edge_e[p][wid] = U[p].e[0];
+      }
+      // odd phase
+#pragma unroll
+      for (uint32_t p = 0; p < NOCC; ++p) {
+        pl[p] = philox_lane(a0, b2, (2u * u + 1u) | (p << 31));
+        sca_first_planes<MODEL, FAST>(hd, pl[p], a.ks, y0[p], y1[p]);
+      }
+      __syncthreads();
+#pragma unroll
+      for (uint32_t p = 0; p < NOCC; ++p) {
+        ScaUnit& x = U[p];
+        uint32_t en = __shfl_down_sync(0xffffffffu, x.e[0], 1);
+        if (last) en = edge_e[p][wid_next];
+        if (p == 0)
+          sca_decide<MODEL, DIS, PQ, COUNT, FAST, 1, 0>(x, en, Q, q_odd, a.rates, kmax, hd, pl[p], y0[p], y1[p], a.ks,
+                                                        cnt, h);
+        else
+          sca_decide<MODEL, DIS, PQ, COUNT, FAST, 1, 1>(x, en, Q, q_odd, a.rates, kmax, hd, pl[p], y0[p], y1[p], a.ks,
+                                                        cnt, h);
+        uint32_t hp = __shfl_up_sync(0xffffffffu, h[3], 1);
+        if (lane == 0u) hp = 0u;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          x.o[g] ^= h[g];
+          x.e[g] ^= odd_flips(h[g], g > 0 ? h[g - 1] : hp);
+        }
+        if (last) edge_c[p][wid] = h[3] >> 31;
+      }
+      if (TURNS) {
+        settle();
+        cnt.c[3] += PQ ? sca_turn_all<1>(U[0], U[NOCC - 1], Q[NQ == 2 ? 1 : 0], u, active, a0, b2, hd[kmax + 1], a)
+                       : sca_turn_pool<1>(U[0], U[NOCC - 1], Q[0], turn[wid], u, active, a0, b2, hd[kmax + 1], a);
+      }
+    }
+    if (rec < a.n_times && a.times[rec] == s0 + it) {
+      if (!TURNS) {
+        settle();
+        clear_edges();
+      }
+#pragma unroll
+      for (uint32_t p = 0; p < NOCC; ++p) {
+        uint32_t x[8];
+        to_words(U[p], x);
+        if (active) store8(lat + p * W + 8u * u, x);
+      }
+      __syncthreads();
+      unsigned long long c64[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        c64[k] = active ? cnt.c[k] : 0u;
+        if (k >= 2) c64[k] = cnt.c[k];  // lane changes: the draws a thread made, whoever's sites they were
+        cnt.c[k] = 0u;
+      }
+      sca_record<NOCC, COUNT>(lat, a, rec, s0 + it, sample, warp_tot, warp_s2, c64);
+      ++rec;
+    }
+  }
+  if (!TURNS) settle();
+#pragma unroll
+  for (uint32_t p = 0; p < NOCC; ++p) {
+    uint32_t x[8];
+    to_words(U[p], x);
+    if (active) store8(state + p * W + 8u * u, x);
+  }
+  if (COUNT) {
+    long long tot[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k)
+      tot[k] = block_sum((active || k >= 2) ? static_cast<long long>(cnt.c[k]) : 0ll, warp_tot);
+    if (threadIdx.x == 0)
+      for (int k = 0; k < 4; ++k) a.counters[4ull * sample + k] += static_cast<uint64_t>(tot[k]);
+  }
+}
+
 // The SCA kernel.  Ring (MODEL 0): one lattice plane, optionally a bimodal
 // class plane (DIS), or the p-class and q-class planes (DIS and PQ).  Two
 // lanes (MODEL 1): planes A and B and, with turning sites (DIS), the turning
@@ -480,7 +684,7 @@ __device__ void sca_record(const uint32_t* lat, const DomainLaunch& a, uint32_t 
 // every step: at most 512 threads then, so the compiler may use up to 128
 // registers.
 template <uint32_t MODEL, bool DIS, bool COUNT, bool FAST2, bool PQ = false>
-__global__ void __launch_bounds__(DIS ? 512 : 1024) k_sca(const DomainLaunch a) {
+__global__ void __launch_bounds__(DIS ? 512 : 1024) k_sca_smem(const DomainLaunch a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ long long warp_tot[32];
   __shared__ unsigned long long warp_s2[32];
@@ -563,14 +767,40 @@ bool sca_fast2(const DomainLaunch& a) {
   return regular(a.rates.p) && regular(a.rates.q) && a.sca_kmax <= 2;
 }
 
+template <typename K>
+cudaError_t launch_sca_kernel(K kernel, const DomainLaunch& a, uint32_t threads, size_t smem, cudaStream_t st) {
+  (void)cudaGetLastError();
+  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (e != cudaSuccess) return e;
+  kernel<<<a.geo.S, threads, smem, st>>>(a);
+  return cudaGetLastError();
+}
+
+// Ring without disorder whose rates are neither 0 nor "always" and take at
+// most two random planes: the specialised comparisons.
+ScaFast sca_fast(const DomainLaunch& a) {
+  const auto regular = [](uint32_t t) { return t != 0u && t != 0xFFFFFFFFu; };
+  if (a.model != kRing || a.dis != kDisNone || !regular(a.rates.p) || !regular(a.rates.q) || a.sca_kmax > 2) return kScaAny;
+  if (a.sca_kmax == 1) return kScaHalf;
+  return ((a.rates.p >> 30) == 2u || (a.rates.q >> 30) == 2u) ? kScaTwoPlanes : kScaQuarters;
+}
+
 template <uint32_t MODEL, bool DIS, bool COUNT, bool FAST2, bool PQ = false>
 cudaError_t launch_sca_t(const DomainLaunch& a, uint32_t threads, size_t smem, cudaStream_t st) {
-  (void)cudaGetLastError();
-  const cudaError_t e = cudaFuncSetAttribute(k_sca<MODEL, DIS, COUNT, FAST2, PQ>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  k_sca<MODEL, DIS, COUNT, FAST2, PQ><<<a.geo.S, threads, smem, st>>>(a);
-  return cudaGetLastError();
+  const uint32_t units = a.geo.W / 8u;
+  if (units <= (DIS ? 512u : 1024u)) {
+    const uint32_t nocc = MODEL == kTwoLane ? 2u : 1u, t = (units + 31u) / 32u * 32u;
+    const size_t sm = 4ull * nocc * a.geo.W + (MODEL == kTwoLane && DIS ? sizeof(ScaTurnScratch) * (t / 32u) : 0u);
+    if constexpr (FAST2) {
+      const ScaFast f = sca_fast(a);
+      if (f == kScaHalf) return launch_sca_kernel(k_sca<MODEL, DIS, COUNT, kScaHalf, PQ>, a, t, sm, st);
+      if (f == kScaQuarters) return launch_sca_kernel(k_sca<MODEL, DIS, COUNT, kScaQuarters, PQ>, a, t, sm, st);
+      return launch_sca_kernel(k_sca<MODEL, DIS, COUNT, kScaTwoPlanes, PQ>, a, t, sm, st);
+    } else {
+      return launch_sca_kernel(k_sca<MODEL, DIS, COUNT, kScaAny, PQ>, a, t, sm, st);
+    }
+  }
+  return launch_sca_kernel(k_sca_smem<MODEL, DIS, COUNT, FAST2, PQ>, a, threads, smem, st);
 }
 
 // ---------------------------------------------------------------------------
