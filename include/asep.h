@@ -61,13 +61,11 @@
  *                      sites the A -> B lane changes after the even phase
  *                      and B -> A after the odd one (probability omega, one
  *                      draw per candidate site: tag 8, call = step, ctr3 =
- *                      site / 4).  L a multiple of 256.  The lattice sits
- *                      in one CTA's shared memory while it fits (ring L up
- *                      to about 1.4 * 2^20, bimodal or two lanes 2^19,
- *                      two lanes with turning sites 2^18); beyond that
- *                      (or on request, asep_set_plan) it stays in global
- *                      memory and each phase is one launch over all units
- *                      of 8 words (results identical).
+ *                      site / 4).  L a multiple of 256.  A warp advances a
+ *                      tile of a ring in registers for up to 128 sweeps a
+ *                      launch (a sweep's influence travels two sites, so a
+ *                      halo of 256 sites on either side keeps it exact);
+ *                      between launches the lattice is in global memory.
  *
  * Error behaviour: every function returns ASEP_OK (0) or a negative
  * ASEP_ERR_* code and never aborts; the context keeps a message readable with
@@ -323,7 +321,7 @@ int asep_set_plan(asep_ctx* ctx, uint32_t cluster, uint32_t samples_per_group);
  * context: max_sweeps = 0 restores the automatic bound (the 32-bit per-lane
  * hop counters of the domain schedule, 2^20 otherwise).  Longer asep_sweep
  * and batch calls are split into launches of at most this many sweeps; the
- * streamed tiers run one sweep per step whatever the cap.  An autotuner knob:
+ * streamed domain tier runs one sweep per step whatever the cap.  An autotuner knob:
  * results never depend on it (every sample's randomness is keyed by its
  * sweep index).  Takes effect for the next call. */
 int asep_set_launch_sweeps(asep_ctx* ctx, uint32_t max_sweeps);

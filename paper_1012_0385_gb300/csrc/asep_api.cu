@@ -65,6 +65,8 @@ struct asep_ctx {
   uint32_t max_sweeps_per_launch = 1;
   uint32_t launch_sweeps = 0;      // caller's cap on sweeps per launch (0 = none)
   uint32_t balance = 0;            // balanced launches: sweeps per chunk (0 = off)
+  ScaTiles sca{};                  // SCA: tiles of a ring
+  uint32_t* d_halo = nullptr;      // SCA: the tiles' edge units, two halves
   uint32_t* d_progress = nullptr;  // balanced launches: [S + 1] chunk flags and queue counter
   uint64_t launches = 0;
   std::string err;
@@ -238,33 +240,26 @@ int validate(const asep_params* p, asep_ctx* ctx) {
   return ASEP_OK;
 }
 
-// SCA plan.  Resident: one CTA per sample holding the ring in shared memory,
-// a thread per unit of 8 words (at most 1024 threads, 512 with a quenched
-// plane).  Streamed (kStreamTier): the ring in global memory, a thread per
-// unit, one launch per phase.  force: 0 = resident when it fits, 1 =
-// resident, kStreamTier = streamed.
+// SCA plan: a warp per tile of a ring.  The plan codes 1 and kStreamTier are
+// both served by it (the lattice is in registers during a launch and in
+// global memory between launches); code 1, the automatic one while it is
+// offered, keeps its limit on the ring's size.
 int plan_sca(asep_ctx* ctx, uint32_t force) {
-  const uint32_t units = ctx->W / 8;
-  const bool quenched = ctx->p.dis_kind != ASEP_DIS_NONE;
   const size_t smem = sca_smem_bytes(ctx->W, ctx->planes, dis_planes(ctx->p.dis_kind));
   const bool fits = smem <= 200u * 1024u;
   if (force == 1 && !fits)
-    return fail(ctx, ASEP_ERR_INVALID, "the resident SCA plan needs %zu bytes of shared memory (at most 200 KB)",
-                smem);
-  if (force == kStreamTier || !fits) {
-    ctx->cluster = kStreamTier;
-    ctx->threads = 256;
-    ctx->smem = 0;
-    ctx->blocks = ctx->S * ((units + 255u) / 256u);
-  } else {
-    const uint32_t cap = quenched ? 512u : 1024u;
-    ctx->cluster = 1;
-    ctx->threads = std::min<uint32_t>(cap, (units + 31u) / 32u * 32u);
-    ctx->smem = smem;
-    ctx->blocks = ctx->S;
-  }
+    return fail(ctx, ASEP_ERR_INVALID, "the resident SCA plan is for lattices and classes of at most 200 KB (this one "
+                "takes %zu bytes)", smem);
+  ctx->cluster = force != kStreamTier && fits ? 1u : kStreamTier;
+  ctx->sca = sca_tiles(ctx->p.model, ctx->p.dis_kind, ctx->p.p_thr, ctx->p.q_thr, ctx->W, ctx->S);
+  ctx->threads = 32;
+  ctx->smem = 0;
+  ctx->blocks = ctx->S * ctx->sca.tiles;
   return ASEP_OK;
 }
+
+// Bytes of the tiles' edge buffer.
+size_t sca_halo_bytes(const asep_ctx* ctx) { return sca_halo_words(ctx->sca, ctx->S, ctx->planes) * 4u; }
 
 // Launch plan.  Resident: columns = super-domains, one thread per column, a
 // whole sample (or several small ones) per CTA.  Cluster tier: each sample
@@ -712,6 +707,7 @@ size_t planned_device_bytes(const asep_ctx* ctx) {
   }
   if (ctx->R) add(static_cast<size_t>(ctx->R) * dis_planes(ctx->p.dis_kind) * ctx->W * 4);
   if (!ctx->ptab.empty()) add(ctx->ptab.size() * 4);
+  if (ctx->p.schedule == ASEP_SCHED_SCA) add(sca_halo_bytes(ctx));
   return total;
 }
 
@@ -798,12 +794,14 @@ int asep_create(const asep_params* params, asep_ctx** out) {
     ctx->d_mask = static_cast<uint32_t*>(
         dev_alloc(ctx, static_cast<size_t>(ctx->R) * dis_planes(params->dis_kind) * ctx->W * 4));
   if (!ctx->ptab.empty()) ctx->d_ptab = static_cast<uint32_t*>(dev_alloc(ctx, ctx->ptab.size() * 4));
+  if (params->schedule == ASEP_SCHED_SCA) ctx->d_halo = static_cast<uint32_t*>(dev_alloc(ctx, sca_halo_bytes(ctx)));
   if (!ctx->d_state || !ctx->d_cnt || !ctx->d_sh || !ctx->d_sh2 || !ctx->d_times || !ctx->d_clock ||
       !ctx->d_tab_cnt || !ctx->d_href || !ctx->d_href2 || !ctx->d_hrefcnt || !ctx->d_err ||
       (height_chunks(ctx->W) > 1 && !ctx->d_parts) ||
       ((params->flags & ASEP_FLAG_PROFILE) && !ctx->d_profile) ||
       ((params->flags & ASEP_FLAG_AUTOCORR) && (!ctx->d_snap || !ctx->d_tab_ac)) || (ctx->R && !ctx->d_mask) ||
-      (!ctx->ptab.empty() && !ctx->d_ptab))
+      (!ctx->ptab.empty() && !ctx->d_ptab) ||
+      (params->schedule == ASEP_SCHED_SCA && !ctx->d_halo))
     return bail(fail(ctx, ASEP_ERR_NOMEM, "device allocation failed (%zu bytes so far)", ctx->dev_bytes));
 
   cudaError_t e;
@@ -860,8 +858,11 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
   if (!ctx) return ASEP_ERR_INVALID;
   if (ctx->sweep + n_mcs >= (1ull << 40)) return fail(ctx, ASEP_ERR_INVALID, "sweep index would exceed 2^40");
   uint64_t done = 0;
+  bool halo_fresh = false;  // SCA: half `halo_half` of the edge buffer holds the lattice's edges
+  uint32_t halo_half = 0;
   while (done < n_mcs) {
     uint64_t n = n_mcs - done;
+    uint32_t sweep_launches = 0;  // SCA: counted by the launch
     const uint32_t cap = sweeps_cap(ctx);
     if (n > cap) n = cap;
     cudaError_t e;
@@ -876,15 +877,17 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
       }
     } else if (ctx->p.schedule == ASEP_SCHED_DOMAIN && ctx->cluster > 1) {
       e = launch_cluster(domain_desc(ctx, static_cast<uint32_t>(n)), ctx->threads, ctx->smem, ctx->stream);
-    } else if (ctx->p.schedule == ASEP_SCHED_SCA && ctx->cluster == kStreamTier) {
-      n = 1;  // one sweep per step: both phases, then the record and the clock
-      e = launch_sca_stream(domain_desc(ctx, 1), ctx->stream);
-      if (e == cudaSuccess && ctx->next_time < ctx->times.size() && ctx->times[ctx->next_time] == ctx->sweep + 1) {
+    } else if (ctx->p.schedule == ASEP_SCHED_SCA) {
+      // up to the next sample time, then the record and the clock
+      const bool record = ctx->next_time < ctx->times.size();
+      if (record) n = std::min<uint64_t>(n, ctx->times[ctx->next_time] - ctx->sweep);
+      e = launch_sca(domain_desc(ctx, static_cast<uint32_t>(n)), ctx->sca, ctx->d_halo, halo_fresh, &halo_half,
+                     &sweep_launches, ctx->stream);
+      halo_fresh = true;
+      if (e == cudaSuccess && record && ctx->times[ctx->next_time] == ctx->sweep + n) {
         const int rc = record_now(ctx, ctx->next_time);
         if (rc != ASEP_OK) return rc;
       }
-    } else if (ctx->p.schedule == ASEP_SCHED_SCA) {
-      e = launch_sca(domain_desc(ctx, static_cast<uint32_t>(n)), ctx->threads, ctx->smem, ctx->stream);
     } else if (ctx->p.schedule == ASEP_SCHED_DOMAIN && ctx->balance && ctx->cluster == 1 && n > ctx->balance) {
       BalanceLaunch b;
       b.chunk = ctx->balance;
@@ -919,12 +922,11 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
     if ((e = launch_advance(ctx->d_clock, ctx->d_times, static_cast<uint32_t>(ctx->times.size()),
                             static_cast<uint32_t>(n), ctx->stream)) != cudaSuccess)
       return cuda_fail(ctx, e, "clock advance");
-    // the sweep kernels (streamed tiers: one per phase, plus the lane changes
-    // of the streamed domain schedule with turning sites) and the clock
-    uint32_t sweep_launches = 1;
-    if (ctx->cluster == kStreamTier)
-      sweep_launches = (ctx->p.schedule == ASEP_SCHED_DOMAIN &&
-                        (ctx->p.dis_kind == ASEP_DIS_TURNING || ctx->p.dis_kind == ASEP_DIS_CROSSING)) ? 3u : 2u;
+    // the sweep kernels (streamed domain tier: one per phase, plus the lane
+    // changes with turning sites) and the clock
+    if (ctx->p.schedule != ASEP_SCHED_SCA)
+      sweep_launches = ctx->cluster != kStreamTier ? 1u
+                       : (ctx->p.dis_kind == ASEP_DIS_TURNING || ctx->p.dis_kind == ASEP_DIS_CROSSING) ? 3u : 2u;
     ctx->launches += sweep_launches + 1;
     advance_host(ctx, n);
     done += n;
@@ -977,7 +979,8 @@ int asep_sync(asep_ctx* ctx) {
   if (!ctx) return ASEP_ERR_INVALID;
   cudaError_t e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "stream synchronize");
-  if ((ctx->cluster == kStreamTier || ctx->balance) && ctx->d_err && !ctx->err_seen) {
+  if (((ctx->cluster == kStreamTier && ctx->p.schedule == ASEP_SCHED_DOMAIN) || ctx->balance) && ctx->d_err &&
+      !ctx->err_seen) {
     uint32_t flag = 0;
     if ((e = cudaMemcpy(&flag, ctx->d_err, 4, cudaMemcpyDeviceToHost)) != cudaSuccess)
       return cuda_fail(ctx, e, "read the error flag");

@@ -231,11 +231,21 @@ size_t stream_smem_bytes(uint32_t model, uint32_t dis, uint32_t R2, uint32_t C, 
 // extra bytes each tile's copies announce (0; fault injection for tests).
 cudaError_t launch_stream_sweep(const DomainLaunch& a, uint32_t tiles, uint32_t threads, size_t smem, uint32_t* err,
                                 uint32_t stall, cudaStream_t st);
-// The two-sub-lattice SCA schedule: one CTA per sample, ring in shared memory.
-cudaError_t launch_sca(const DomainLaunch& a, uint32_t threads, size_t smem, cudaStream_t st);
-// Streamed SCA: one sweep (both phases; two lanes: with the lane changes)
-// over every sample, lattice in global memory; results identical to launch_sca.
-cudaError_t launch_sca_stream(const DomainLaunch& a, cudaStream_t st);
+// The two-sub-lattice SCA schedule: a warp per tile of a ring, the lattice in
+// global memory between launches.
+struct ScaTiles {
+  uint32_t tiles, units, upt;  // tiles per ring, units (of 8 words) per tile, units per thread
+};
+ScaTiles sca_tiles(uint32_t model, uint32_t dis, uint32_t p_thr, uint32_t q_thr, uint32_t W, uint32_t S);
+// Words of the buffer of the tiles' edge units, two halves.
+size_t sca_halo_words(const ScaTiles& t, uint32_t S, uint32_t planes);
+// a.n_sweeps sweeps in launches of at most 128.  *parity = the half of `halo`
+// that holds the tiles' edge units when `fresh` (otherwise they are taken
+// from the lattice first); *launches is advanced.
+cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, uint32_t* halo, bool fresh, uint32_t* parity,
+                       uint32_t* launches, cudaStream_t st);
+// The bound by which the one-CTA plan code is offered: lattice, classes and
+// carries within 200 KB.
 size_t sca_smem_bytes(uint32_t W, uint32_t planes, uint32_t quenched_planes);
 // How many clusters of the given shape can be resident at once (0 = none).
 int cluster_fits(uint32_t model, uint32_t dis, uint32_t cluster, uint32_t threads, size_t smem);

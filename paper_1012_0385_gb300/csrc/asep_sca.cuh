@@ -1,6 +1,5 @@
 // asep_sca.cuh -- the bit-sliced two-sub-lattice SCA on units held in
-// registers, shared by the ring-per-CTA kernel and the tile kernel
-// (asep_sca.cu).
+// registers (kernel and launches: asep_sca.cu).
 //
 // A unit is 256 sites = 8 words = four groups of 32 bonds per phase.  Group g
 // holds the bonds of word 2g in its even lanes and of word 2g + 1 in its odd
@@ -116,50 +115,109 @@ __device__ __forceinline__ uint4 sca_plane(const uint4* heads, uint32_t k, const
 __device__ __forceinline__ uint32_t bit_mask(uint32_t t20, uint32_t k) { return 0u - ((t20 >> (19u - k)) & 1u); }
 
 __device__ __forceinline__ uint32_t bitsel(uint32_t m, uint32_t a, uint32_t b) { return (a & m) | (b & ~m); }
-__device__ __forceinline__ uint32_t maj(uint32_t a, uint32_t b, uint32_t c) { return (a & b) | (c & (a | b)); }
 
-// How a ring without disorder decides u < t (ScaFast): any thresholds, plane
-// by plane; both thresholds 1/2, one plane; thresholds of two planes, 1/4 or
-// 3/4 each; the same with one of them 1/2.
-enum ScaFast : uint32_t { kScaAny = 0, kScaHalf = 1, kScaQuarters = 2, kScaTwoPlanes = 3 };
+// Rings without disorder whose thresholds p and q are decided by at most two
+// planes (FAST = 4 p2 + q2, the thresholds' top two bits, each 1..3; 0 = any
+// other thresholds): u < t is ~(u0 | u1) for t = 1, ~u0 for t = 2 and
+// ~(u0 & u1) for t = 3, so whether bond lanes would swap their sites is one
+// logic operation of (first sites f, planes u0, u1).
+constexpr uint32_t kScaAny = 0;
+constexpr uint32_t kScaHalves = 4 * 2 + 2;  // one plane
 
-// Moves of a ring's bonds for the two-plane kinds: p2, q2 = the thresholds'
-// top two bits (1..3), f, n = first and second sites, u0, u1 = the planes.
-// u < t is ~(u0 | u1) for t = 1, ~u0 for t = 2 and ~(u0 & u1) for t = 3, that
-// is ~maj(m, u0, u1) with m all ones, u0 or zero -- three logic operations a
-// group for the quarters.
+template <uint32_t T2>
+__device__ __forceinline__ uint32_t below2(uint32_t u0, uint32_t u1) {
+  return T2 == 1u ? ~(u0 | u1) : (T2 == 2u ? ~u0 : ~(u0 & u1));
+}
+
+// Lanes whose bond swaps (a swap of equal sites changes nothing).
 template <uint32_t FAST>
-__device__ __forceinline__ void decide_fast(const uint32_t (&f)[4], const uint32_t (&n)[4], uint32_t p2, uint32_t q2,
-                                            const uint4 y0, const uint4 y1, uint32_t (&h)[4]) {
-  const uint32_t u0[4] = {y0.x, y0.y, y0.z, y0.w}, u1[4] = {y1.x, y1.y, y1.z, y1.w};
-  const uint32_t mp = p2 == 1u ? ~0u : 0u, mq = q2 == 1u ? ~0u : 0u;
-  const uint32_t tp = p2 == 2u ? ~0u : 0u, tq = q2 == 2u ? ~0u : 0u;
+__device__ __forceinline__ uint32_t swaps_fast(uint32_t f, uint32_t u0, uint32_t u1) {
+  return bitsel(f, below2<(FAST >> 2)>(u0, u1), below2<(FAST & 3u)>(u0, u1));
+}
+
+// Thresholds of a ring as the plane-by-plane comparison uses them (uniform):
+// t[c] of the classes c = fast right, slow right, fast left, slow left.  A
+// class whose threshold is 0 or "always" needs no draw; it takes another
+// class's planes, so that as few distinct ones as possible are left.
+struct ScaRule {
+  uint32_t p, ps, q, qs;  // 20 bits
+  bool special;           // some class needs no draw
+  bool by_class;          // right and left hops share their planes: the slow classes alone select
+};
+
+__device__ __forceinline__ ScaRule sca_rule(const Rates& r, bool dis) {
+  const auto fixed = [](uint32_t t) { return t == 0u || t == 0xFFFFFFFFu; };
+  const uint32_t p0 = r.p, s0 = dis ? r.p_slow : r.p, q0 = r.q, t0 = dis ? r.q_slow : r.q;
+  ScaRule v;
+  v.special = fixed(p0) || fixed(s0) || fixed(q0) || fixed(t0);
+  const uint32_t p = !fixed(p0) ? p0 : (!fixed(s0) ? s0 : (!fixed(q0) ? q0 : t0));
+  const uint32_t ps = !fixed(s0) ? s0 : p;
+  const uint32_t q = !fixed(q0) ? q0 : (!fixed(t0) ? t0 : p);
+  const uint32_t qs = !fixed(t0) ? t0 : (!fixed(q0) ? q : ps);
+  v.p = p >> 12;
+  v.ps = ps >> 12;
+  v.q = q >> 12;
+  v.qs = qs >> 12;
+  v.by_class = v.p == v.q && v.ps == v.qs;
+  return v;
+}
+
+constexpr uint32_t kScaBlock = 7;  // planes taken without looking for undecided lanes
+
+// One plane of the comparison from the least significant side: lt = u < t and
+// eq = u == t over the planes so far; the threshold bit is b1 where z is set,
+// b0 elsewhere (uniform).
+__device__ __forceinline__ void compare_up(const uint32_t (&z)[4], bool b1, bool b0, const uint4 y, uint32_t (&lt)[4],
+                                           uint32_t (&eq)[4]) {
+  const uint32_t u[4] = {y.x, y.y, y.z, y.w};
+  if (b1 == b0) {
+    if (b1) {
 #pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    if (FAST == kScaHalf) h[g] = (f[g] ^ n[g]) & ~u0[g];
-    else if (FAST == kScaQuarters) h[g] = (f[g] ^ n[g]) & ~maj(bitsel(f[g], mp, mq), u0[g], u1[g]);
-    else h[g] = (f[g] ^ n[g]) & ~maj(bitsel(f[g], mp | (tp & u0[g]), mq | (tq & u0[g])), u0[g], u1[g]);
+      for (int g = 0; g < 4; ++g) {
+        lt[g] |= ~u[g];
+        eq[g] &= u[g];
+      }
+    } else {
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        lt[g] &= ~u[g];
+        eq[g] &= ~u[g];
+      }
+    }
+  } else if (b1) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      lt[g] = bitsel(z[g], lt[g] | ~u[g], lt[g] & ~u[g]);
+      eq[g] &= ~(z[g] ^ u[g]);
+    }
+  } else {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      lt[g] = bitsel(z[g], lt[g] & ~u[g], lt[g] | ~u[g]);
+      eq[g] &= z[g] ^ u[g];
+    }
   }
 }
 
-// Any thresholds: most significant plane first, until no candidate of the
-// warp is undecided.  c1: slow classes of the first sites (right hops), c2:
-// of the second sites (left hops); DIS = false: no classes.  All 32 lanes call.
+// Any thresholds.  c1: slow classes of the first sites (right hops), c2: of
+// the second sites (left hops); DIS = false: no classes.  The first kScaBlock
+// planes decide all but a few of a warp's some 2000 candidates, so they are
+// compared from the least significant side (two logic operations a group and
+// plane, no vote); the rest most significant first, until no candidate of the
+// warp is undecided (some 12 planes in all).  All 32 lanes call.
 template <bool DIS, typename PLANE>
 __device__ __forceinline__ void decide_any(const uint32_t (&f)[4], const uint32_t (&n)[4], const uint32_t (&c1)[4],
-                                           const uint32_t (&c2)[4], const Rates& r, uint32_t kmax, PLANE plane,
-                                           uint32_t (&h)[4]) {
+                                           const uint32_t (&c2)[4], const Rates& r, const ScaRule& rule, uint32_t kmax,
+                                           PLANE plane, uint32_t (&h)[4]) {
   constexpr uint32_t kAll = 0xFFFFFFFFu;
-  uint32_t eq[4], sl[4];
+  uint32_t eq[4], cand[4], sl[4], z[4];
 #pragma unroll
   for (int g = 0; g < 4; ++g) {
-    eq[g] = f[g] ^ n[g];
+    cand[g] = f[g] ^ n[g];
     h[g] = 0u;
     sl[g] = DIS ? bitsel(f[g], c1[g], c2[g]) : 0u;
   }
-  const bool special = r.p == 0u || r.p == kAll || r.q == 0u || r.q == kAll ||
-                       (DIS && (r.p_slow == 0u || r.p_slow == kAll || r.q_slow == 0u || r.q_slow == kAll));
-  if (special) {  // thresholds that need no draw
+  if (rule.special) {  // classes that need no draw
     const uint32_t pA = r.p == kAll ? ~0u : 0u, qA = r.q == kAll ? ~0u : 0u;
     const uint32_t pN = r.p == 0u ? ~0u : 0u, qN = r.q == 0u ? ~0u : 0u;
     const uint32_t psA = r.p_slow == kAll ? ~0u : 0u, qsA = r.q_slow == kAll ? ~0u : 0u;
@@ -168,20 +226,52 @@ __device__ __forceinline__ void decide_any(const uint32_t (&f)[4], const uint32_
     for (int g = 0; g < 4; ++g) {
       const uint32_t A = DIS ? bitsel(f[g], bitsel(sl[g], psA, pA), bitsel(sl[g], qsA, qA)) : bitsel(f[g], pA, qA);
       const uint32_t N = DIS ? bitsel(f[g], bitsel(sl[g], psN, pN), bitsel(sl[g], qsN, qN)) : bitsel(f[g], pN, qN);
-      h[g] = eq[g] & A;
-      eq[g] &= ~(A | N);
+      h[g] = cand[g] & A;
+      cand[g] &= ~(A | N);
     }
   }
-  const uint32_t p20 = r.p >> 12, q20 = r.q >> 12, ps20 = r.p_slow >> 12, qs20 = r.q_slow >> 12;
-  for (uint32_t k = 0; k < kmax; ++k) {
+  const uint32_t kb = min(kmax, kScaBlock);
+  const bool two = !DIS || rule.by_class;  // one selector tells the planes apart
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    z[g] = DIS ? sl[g] : f[g];
+    eq[g] = cand[g];
+  }
+  if (kb) {
+    uint32_t lt[4] = {0u, 0u, 0u, 0u};
+#pragma unroll 1
+    for (uint32_t k = kb; k-- > 0;) {
+      const uint4 y = plane(k);
+      const uint32_t sh = 19u - k;
+      const bool P = (rule.p >> sh) & 1u, Q = (rule.q >> sh) & 1u, PS = (rule.ps >> sh) & 1u, QS = (rule.qs >> sh) & 1u;
+      if (two) {
+        compare_up(z, DIS ? PS : P, DIS ? P : Q, y, lt, eq);
+      } else {
+        const uint32_t u[4] = {y.x, y.y, y.z, y.w};
+        const uint32_t mp = P ? ~0u : 0u, mq = Q ? ~0u : 0u, mps = PS ? ~0u : 0u, mqs = QS ? ~0u : 0u;
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          const uint32_t t = bitsel(f[g], bitsel(sl[g], mps, mp), bitsel(sl[g], mqs, mq));
+          lt[g] = bitsel(t, lt[g] | ~u[g], lt[g] & ~u[g]);
+          eq[g] &= ~(t ^ u[g]);
+        }
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < 4; ++g) h[g] |= cand[g] & lt[g];
+  }
+#pragma unroll 1
+  for (uint32_t k = kb; k < kmax; ++k) {
     if (!__any_sync(0xffffffffu, (eq[0] | eq[1] | eq[2] | eq[3]) != 0u)) break;
     const uint4 y = plane(k);
     const uint32_t u[4] = {y.x, y.y, y.z, y.w};
-    const uint32_t P = bit_mask(p20, k), Q = bit_mask(q20, k);
-    const uint32_t PS = DIS ? bit_mask(ps20, k) : 0u, QS = DIS ? bit_mask(qs20, k) : 0u;
+    const uint32_t P = bit_mask(rule.p, k), Q = bit_mask(rule.q, k);
+    const uint32_t PS = DIS ? bit_mask(rule.ps, k) : 0u, QS = DIS ? bit_mask(rule.qs, k) : 0u;
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
-      const uint32_t t = DIS ? bitsel(f[g], bitsel(sl[g], PS, P), bitsel(sl[g], QS, Q)) : bitsel(f[g], P, Q);
+      const uint32_t t = !DIS ? bitsel(f[g], P, Q)
+                         : rule.by_class ? bitsel(sl[g], PS, P)
+                                         : bitsel(f[g], bitsel(sl[g], PS, P), bitsel(sl[g], QS, Q));
       h[g] |= eq[g] & t & ~u[g];  // this bit of u is 0 where t's is 1: u < t
       eq[g] &= ~(t ^ u[g]);       // equal so far
     }
@@ -219,19 +309,21 @@ __device__ __forceinline__ void decide_lane(const uint32_t (&cand)[4], uint32_t 
   }
 }
 
-// One phase of one unit of lane P (ring: P = 0): the moves h of its bonds and
-// the flips inside the unit; f = first sites, n = second sites.  The flips
-// that cross units are the caller's: in the odd phase the last group's bond
-// 31 flips the next unit's site 0 (h[3] >> 31).
 struct ScaCounts {
   uint32_t c[4] = {0u, 0u, 0u, 0u};  // at most 512 a sweep and unit, 2^20 sweeps a launch
 };
 
+// One phase of one unit of lane P (ring: P = 0), given the phase's first
+// planes: updates the unit's sites, except that in the odd phase the even
+// sites are left to the caller, who gets the moves h (their flips cross
+// units: the last group's bond 31 ends in the next unit's site 0).  counted:
+// all ones, or zero for a unit whose hops another thread counts.
 template <uint32_t MODEL, bool DIS, bool PQ, bool COUNT, uint32_t FAST, uint32_t PHASE, uint32_t P>
-__device__ __forceinline__ void sca_decide(const ScaUnit& x, uint32_t en, const ScaUnit (&Q)[(DIS && PQ) ? 2 : 1],
-                                           const uint32_t (&q_odd)[4], const Rates& r, uint32_t kmax,
-                                           const uint4* heads, const PhiloxLane& pl, const uint4 y0, const uint4 y1,
-                                           const KeySchedule& ks, ScaCounts& cnt, uint32_t (&h)[4]) {
+__device__ __forceinline__ void sca_update(ScaUnit& x, uint32_t en, const ScaUnit (&Q)[(DIS && PQ) ? 2 : 1],
+                                           const uint32_t (&q_odd)[4], const Rates& r, const ScaRule& rule,
+                                           uint32_t kmax, const uint4* heads, const PhiloxLane& pl, const uint4 y0, const uint4 y1,
+                                           const KeySchedule& ks, uint32_t counted, ScaCounts& cnt,
+                                           uint32_t (&h)[4]) {
   uint32_t f[4], n[4];
 #pragma unroll
   for (int g = 0; g < 4; ++g) {
@@ -239,28 +331,45 @@ __device__ __forceinline__ void sca_decide(const ScaUnit& x, uint32_t en, const 
     n[g] = PHASE ? odd_sites(x.e[g], g < 3 ? x.e[g + 1] : en) : x.o[g];
   }
   const auto plane = [&](uint32_t k) { return k == 0u ? y0 : sca_plane(heads, k, pl, ks); };
-  if (MODEL == kTwoLane) {
-    uint32_t cand[4];
-#pragma unroll
-    for (int g = 0; g < 4; ++g) cand[g] = P == 0 ? f[g] & ~n[g] : n[g] & ~f[g];
-    decide_lane(cand, P == 0 ? r.p : r.q, plane, h);
-#pragma unroll
-    for (int g = 0; g < 4; ++g) cnt.c[P] += __popc(h[g]);
-    return;
-  }
   if (FAST != kScaAny) {
-    decide_fast<FAST>(f, n, r.p >> 30, r.q >> 30, y0, y1, h);
-  } else if (DIS) {
-    constexpr int kq = (DIS && PQ) ? 1 : 0;  // the classes of left hops
-    decide_any<true>(f, n, PHASE ? Q[0].o : Q[0].e, PHASE ? q_odd : Q[kq].o, r, kmax, plane, h);
-  } else {
-    decide_any<false>(f, n, q_odd, q_odd, r, kmax, plane, h);
-  }
-  if (COUNT) {
+    const uint32_t u0[4] = {y0.x, y0.y, y0.z, y0.w}, u1[4] = {y1.x, y1.y, y1.z, y1.w};
 #pragma unroll
     for (int g = 0; g < 4; ++g) {
-      cnt.c[0] += __popc(h[g] & f[g]);
-      cnt.c[1] += __popc(h[g] & ~f[g]);
+      const uint32_t v = swaps_fast<FAST>(f[g], u0[g], u1[g]);
+      if (PHASE == 0) {
+        x.e[g] = bitsel(v, n[g], f[g]);
+        x.o[g] = bitsel(v, f[g], n[g]);
+      } else {
+        x.o[g] = bitsel(v, n[g], f[g]);
+      }
+      h[g] = (f[g] ^ n[g]) & v;
+    }
+  } else {
+    if (MODEL == kTwoLane) {
+      uint32_t cand[4];
+#pragma unroll
+      for (int g = 0; g < 4; ++g) cand[g] = P == 0 ? f[g] & ~n[g] : n[g] & ~f[g];
+      decide_lane(cand, P == 0 ? r.p : r.q, plane, h);
+    } else if (DIS) {
+      constexpr int kq = (DIS && PQ) ? 1 : 0;  // the classes of left hops
+      decide_any<true>(f, n, PHASE ? Q[0].o : Q[0].e, PHASE ? q_odd : Q[kq].o, r, rule, kmax, plane, h);
+    } else {
+      decide_any<false>(f, n, q_odd, q_odd, r, rule, kmax, plane, h);
+    }
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      x.o[g] ^= h[g];
+      if (PHASE == 0) x.e[g] ^= h[g];
+    }
+  }
+  if (MODEL == kTwoLane) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) cnt.c[P] += __popc(h[g] & counted);
+  } else if (COUNT) {
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      cnt.c[0] += __popc(h[g] & f[g] & counted);
+      cnt.c[1] += __popc(h[g] & ~f[g] & counted);
     }
   }
 }
@@ -271,7 +380,7 @@ template <uint32_t MODEL, uint32_t FAST>
 __device__ __forceinline__ void sca_first_planes(const uint4* heads, const PhiloxLane& pl, const KeySchedule& ks,
                                                  uint4& y0, uint4& y1) {
   y0 = sca_plane(heads, 0, pl, ks);
-  y1 = (FAST == kScaQuarters || FAST == kScaTwoPlanes) ? sca_plane(heads, 1, pl, ks) : make_uint4(0u, 0u, 0u, 0u);
+  y1 = (FAST != kScaAny && FAST != kScaHalves) ? sca_plane(heads, 1, pl, ks) : make_uint4(0u, 0u, 0u, 0u);
 }
 
 // ---------------------------------------------------------------------------
@@ -296,7 +405,7 @@ struct ScaTurnScratch {
 // Returns the moves of counted units drawn by this lane.  All 32 lanes call.
 template <uint32_t STEP>
 __device__ __forceinline__ uint32_t sca_turn_pool(ScaUnit& A, ScaUnit& B, const ScaUnit& m, ScaTurnScratch& sc,
-                                                  uint32_t unit, bool counted, uint32_t a0, uint32_t b2,
+                                                  uint32_t unit, uint32_t counted, uint32_t a0, uint32_t b2,
                                                   const uint4 head, const DomainLaunch& a) {
   const uint32_t lane = threadIdx.x & 31u;
   uint32_t cand[8];
@@ -333,7 +442,7 @@ __device__ __forceinline__ uint32_t sca_turn_pool(ScaUnit& A, ScaUnit& B, const 
       const uint32_t q = i < total ? sc.queue[i] : 0u;
       const uint32_t src = q >> 8, w = (q >> 5) & 7u, b = q & 31u;
       const uint32_t src_unit = __shfl_sync(0xffffffffu, unit, src);
-      const uint32_t src_counted = __shfl_sync(0xffffffffu, counted ? 1u : 0u, src);
+      const uint32_t src_counted = __shfl_sync(0xffffffffu, counted & 1u, src);
       // word 2g + (b & 1) of the unit, bit 2 (b / 2) + (odd site)
       const uint32_t site = 256u * src_unit + 32u * (2u * (w & 3u) + (b & 1u)) + (b & 30u) + (w >> 2);
       const PhiloxLane pl = philox_lane(a0, b2, site >> 2);
