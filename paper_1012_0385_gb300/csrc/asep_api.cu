@@ -67,6 +67,8 @@ struct asep_ctx {
   uint32_t balance = 0;            // balanced launches: sweeps per chunk (0 = off)
   ScaTiles sca{};                  // SCA: tiles of a ring
   uint32_t* d_halo = nullptr;      // SCA: the tiles' edge units, two halves
+  uint32_t sca_records = 0;        // SCA: records a launch holds at most
+  ScaPart* d_sca_parts = nullptr;  // SCA: the tiles' parts of a launch's records
   uint32_t* d_progress = nullptr;  // balanced launches: [S + 1] chunk flags and queue counter
   uint64_t launches = 0;
   std::string err;
@@ -252,6 +254,7 @@ int plan_sca(asep_ctx* ctx, uint32_t force) {
                 "takes %zu bytes)", smem);
   ctx->cluster = force != kStreamTier && fits ? 1u : kStreamTier;
   ctx->sca = sca_tiles(ctx->p.model, ctx->p.dis_kind, ctx->p.p_thr, ctx->p.q_thr, ctx->W, ctx->S);
+  ctx->sca_records = sca_max_records(ctx->times.data(), ctx->times.size(), ctx->S, ctx->sca.tiles, ctx->planes);
   ctx->threads = 32;
   ctx->smem = 0;
   ctx->blocks = ctx->S * ctx->sca.tiles;
@@ -260,6 +263,12 @@ int plan_sca(asep_ctx* ctx, uint32_t force) {
 
 // Bytes of the tiles' edge buffer.
 size_t sca_halo_bytes(const asep_ctx* ctx) { return sca_halo_words(ctx->sca, ctx->S, ctx->planes) * 4u; }
+
+// Bytes of the tiles' parts of a launch's records (none without sample times).
+size_t sca_parts_bytes(const asep_ctx* ctx) {
+  if (!ctx->sca_records) return 0;
+  return (ctx->sca_records + static_cast<size_t>(1)) * ctx->S * ctx->sca.tiles * ctx->planes * sizeof(ScaPart);
+}
 
 // Launch plan.  Resident: columns = super-domains, one thread per column, a
 // whole sample (or several small ones) per CTA.  Cluster tier: each sample
@@ -707,7 +716,10 @@ size_t planned_device_bytes(const asep_ctx* ctx) {
   }
   if (ctx->R) add(static_cast<size_t>(ctx->R) * dis_planes(ctx->p.dis_kind) * ctx->W * 4);
   if (!ctx->ptab.empty()) add(ctx->ptab.size() * 4);
-  if (ctx->p.schedule == ASEP_SCHED_SCA) add(sca_halo_bytes(ctx));
+  if (ctx->p.schedule == ASEP_SCHED_SCA) {
+    add(sca_halo_bytes(ctx));
+    add(sca_parts_bytes(ctx));
+  }
   return total;
 }
 
@@ -794,14 +806,17 @@ int asep_create(const asep_params* params, asep_ctx** out) {
     ctx->d_mask = static_cast<uint32_t*>(
         dev_alloc(ctx, static_cast<size_t>(ctx->R) * dis_planes(params->dis_kind) * ctx->W * 4));
   if (!ctx->ptab.empty()) ctx->d_ptab = static_cast<uint32_t*>(dev_alloc(ctx, ctx->ptab.size() * 4));
-  if (params->schedule == ASEP_SCHED_SCA) ctx->d_halo = static_cast<uint32_t*>(dev_alloc(ctx, sca_halo_bytes(ctx)));
+  if (params->schedule == ASEP_SCHED_SCA) {
+    ctx->d_halo = static_cast<uint32_t*>(dev_alloc(ctx, sca_halo_bytes(ctx)));
+    ctx->d_sca_parts = static_cast<ScaPart*>(dev_alloc(ctx, sca_parts_bytes(ctx)));
+  }
   if (!ctx->d_state || !ctx->d_cnt || !ctx->d_sh || !ctx->d_sh2 || !ctx->d_times || !ctx->d_clock ||
       !ctx->d_tab_cnt || !ctx->d_href || !ctx->d_href2 || !ctx->d_hrefcnt || !ctx->d_err ||
       (height_chunks(ctx->W) > 1 && !ctx->d_parts) ||
       ((params->flags & ASEP_FLAG_PROFILE) && !ctx->d_profile) ||
       ((params->flags & ASEP_FLAG_AUTOCORR) && (!ctx->d_snap || !ctx->d_tab_ac)) || (ctx->R && !ctx->d_mask) ||
       (!ctx->ptab.empty() && !ctx->d_ptab) ||
-      (params->schedule == ASEP_SCHED_SCA && !ctx->d_halo))
+      (params->schedule == ASEP_SCHED_SCA && (!ctx->d_halo || !ctx->d_sca_parts)))
     return bail(fail(ctx, ASEP_ERR_NOMEM, "device allocation failed (%zu bytes so far)", ctx->dev_bytes));
 
   cudaError_t e;
@@ -858,13 +873,12 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
   if (!ctx) return ASEP_ERR_INVALID;
   if (ctx->sweep + n_mcs >= (1ull << 40)) return fail(ctx, ASEP_ERR_INVALID, "sweep index would exceed 2^40");
   uint64_t done = 0;
-  bool halo_fresh = false;  // SCA: half `halo_half` of the edge buffer holds the lattice's edges
-  uint32_t halo_half = 0;
   while (done < n_mcs) {
     uint64_t n = n_mcs - done;
     uint32_t sweep_launches = 0;  // SCA: counted by the launch
     const uint32_t cap = sweeps_cap(ctx);
-    if (n > cap) n = cap;
+    if (ctx->p.schedule == ASEP_SCHED_SCA) n = std::min<uint64_t>(n, 1u << 20);  // split into launches there
+    else if (n > cap) n = cap;
     cudaError_t e;
     if (ctx->p.schedule == ASEP_SCHED_DOMAIN && ctx->cluster == kStreamTier) {
       // one sweep per step: both phases, lane changes, the record, the clock
@@ -878,16 +892,15 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
     } else if (ctx->p.schedule == ASEP_SCHED_DOMAIN && ctx->cluster > 1) {
       e = launch_cluster(domain_desc(ctx, static_cast<uint32_t>(n)), ctx->threads, ctx->smem, ctx->stream);
     } else if (ctx->p.schedule == ASEP_SCHED_SCA) {
-      // up to the next sample time, then the record and the clock
-      const bool record = ctx->next_time < ctx->times.size();
-      if (record) n = std::min<uint64_t>(n, ctx->times[ctx->next_time] - ctx->sweep);
-      e = launch_sca(domain_desc(ctx, static_cast<uint32_t>(n)), ctx->sca, ctx->d_halo, halo_fresh, &halo_half,
-                     &sweep_launches, ctx->stream);
-      halo_fresh = true;
-      if (e == cudaSuccess && record && ctx->times[ctx->next_time] == ctx->sweep + n) {
-        const int rc = record_now(ctx, ctx->next_time);
-        if (rc != ASEP_OK) return rc;
-      }
+      ScaRun run;
+      run.halo = ctx->d_halo;
+      run.parts = ctx->d_sca_parts;
+      run.max_records = ctx->sca_records;
+      run.max_sweeps = cap;
+      run.sweep = ctx->sweep;
+      run.times = ctx->times.data() + ctx->next_time;
+      run.n_times = ctx->times.size() - ctx->next_time;
+      e = launch_sca(domain_desc(ctx, static_cast<uint32_t>(n)), ctx->sca, run, ctx->stream, &sweep_launches);
     } else if (ctx->p.schedule == ASEP_SCHED_DOMAIN && ctx->balance && ctx->cluster == 1 && n > ctx->balance) {
       BalanceLaunch b;
       b.chunk = ctx->balance;

@@ -239,11 +239,30 @@ struct ScaTiles {
 ScaTiles sca_tiles(uint32_t model, uint32_t dis, uint32_t p_thr, uint32_t q_thr, uint32_t W, uint32_t S);
 // Words of the buffer of the tiles' edge units, two halves.
 size_t sca_halo_words(const ScaTiles& t, uint32_t S, uint32_t planes);
-// a.n_sweeps sweeps in launches of at most 128.  *parity = the half of `halo`
-// that holds the tiles' edge units when `fresh` (otherwise they are taken
-// from the lattice first); *launches is advanced.
-cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, uint32_t* halo, bool fresh, uint32_t* parity,
-                       uint32_t* launches, cudaStream_t st);
+// A tile's part of a record: height change and sums of its heights relative
+// to its entry height, autocorrelation overlap, and (plane 0) its hops since
+// the launch began.
+struct ScaPart {
+  int32_t tot, ov;
+  int64_t s1;
+  uint64_t s2;
+  uint32_t hops[4];
+};
+// Records one launch holds at most: as many as fall into it, within 64 MB.
+uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t tiles, uint32_t planes);
+// One call's buffers and schedule (host).
+struct ScaRun {
+  uint32_t* halo;          // sca_halo_words words
+  ScaPart* parts;          // [max_records + 1][S][tiles][planes]
+  uint32_t max_records, max_sweeps;  // per launch
+  uint64_t sweep;          // sweep count at the start of the call
+  const uint64_t* times;   // the sample times not yet recorded
+  size_t n_times;
+};
+// a.n_sweeps sweeps in launches of at most 128, with the records inside them;
+// *launches is advanced.
+cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, const ScaRun& run, cudaStream_t st,
+                       uint32_t* launches);
 // The bound by which the one-CTA plan code is offered: lattice, classes and
 // carries within 200 KB.
 size_t sca_smem_bytes(uint32_t W, uint32_t planes, uint32_t quenched_planes);

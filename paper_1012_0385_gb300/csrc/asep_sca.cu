@@ -45,8 +45,10 @@ constexpr uint64_t kScaManyTiles = 152u * 108u;
 struct ScaTileLaunch {
   uint32_t tiles, units;  // per ring: tiles, units per tile (the last may hold fewer)
   uint32_t n, offset;     // sweeps of this launch, and before it since the context clock
+  uint32_t n_rec, rec_offset;  // sample times inside this launch, and before it since the clock's cursor
   const uint32_t* halo_in;   // [S][tiles][first, last unit][planes][8]
   uint32_t* halo_out;
+  ScaPart* parts;         // [n_rec + 1][S][tiles][planes] (the last entry: the launch's hops)
 };
 
 // ---------------------------------------------------------------------------
@@ -71,6 +73,86 @@ struct ScaTileLaunch {
 // p = 0.75, q = 0.25 1.90 -> 1.65, 201 rings of 391 units with independent
 // classes 13.0 -> 8.6, 128 pairs of lanes of 2^16 with turning sites 6.35 ->
 // 6.5, 2 rings of 2^22 10.3 -> 0.60, 8 rings of 2^28 189 -> 87.
+//
+// Records are taken inside the launch: a tile leaves the sums of its heights
+// relative to its entry height, its height change and its hops so far, and
+// k_sca_records combines the tiles of every record of the launch.  (A record
+// between launches -- the launch, k_heights, the clock, the next launch --
+// took some 25 us; 256 rings of 2^17 with 88 log-spaced records in 2048
+// sweeps spent 2.2 of 5.6 ms there.)
+
+// The tile's hops since the launch began.
+__device__ __forceinline__ void tile_hops(const ScaCounts& cnt, ScaPart* part) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint32_t v = __reduce_add_sync(0xffffffffu, cnt.c[k]);
+    if ((threadIdx.x & 31u) == 31u) part->hops[k] = v;
+  }
+}
+
+// One record of one tile: the other observables, and its part of the height sums.
+template <uint32_t NOCC, uint32_t UPT>
+__device__ void tile_record(const ScaUnit (&U)[NOCC][UPT], const uint32_t (&gu)[UPT], const uint32_t (&counted)[UPT],
+                            const DomainLaunch& a, uint32_t sample, uint64_t time, ScaPart* part, bool count,
+                            const ScaCounts& cnt) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const Extras& ex = a.ex;
+#pragma unroll
+  for (uint32_t p = 0; p < NOCC; ++p) {
+    int tot = 0, ov = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < UPT; ++j) {
+      if (!counted[j]) continue;
+      uint32_t x[8];
+      to_words(U[p][j], x);
+      const size_t base = (static_cast<size_t>(sample) * NOCC + p) * a.geo.W + 8u * gu[j];
+#pragma unroll
+      for (int w = 0; w < 8; ++w) {
+        const int ones = __popc(x[w]);
+        tot += 2 * ones - 32;
+        if (ex.profile) ex.profile[base + w] += ones;
+        if (ex.snap) {
+          if (time == ex.t0) ex.snap[base + w] = x[w];
+          if (time >= ex.t0) ov += __popc(time == ex.t0 ? x[w] : x[w] & ex.snap[base + w]);
+        }
+      }
+    }
+    int incl = tot;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, d);
+      if (lane >= static_cast<uint32_t>(d)) incl += v;
+    }
+    long long h = incl - tot, s1 = 0;
+    unsigned long long s2 = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < UPT; ++j) {
+      if (!counted[j]) continue;
+      uint32_t x[8];
+      to_words(U[p][j], x);
+#pragma unroll 1
+      for (int w = 0; w < 8; ++w) {
+        add_word_heights(x[0], h, s1, s2);
+#pragma unroll
+        for (int v = 0; v < 7; ++v) x[v] = x[v + 1];
+      }
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      s1 += __shfl_xor_sync(0xffffffffu, s1, d);
+      s2 += __shfl_xor_sync(0xffffffffu, s2, d);
+      ov += __shfl_xor_sync(0xffffffffu, ov, d);
+    }
+    if (lane == 31u) {
+      part[p].tot = incl;
+      part[p].ov = ov;
+      part[p].s1 = s1;
+      part[p].s2 = s2;
+    }
+  }
+  if (count) tile_hops(cnt, part);
+}
+
 template <uint32_t MODEL, bool DIS, bool COUNT, uint32_t FAST, bool PQ, uint32_t UPT>
 __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
     k_sca_tile(const DomainLaunch a, const ScaTileLaunch t) {
@@ -140,13 +222,23 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
   }
 
   ScaCounts cnt;
-  for (uint32_t base = 0; base < t.n; base += chunk) {
-    const uint32_t len = min(chunk, t.n - base);
-    __syncwarp();
-    sca_fill_heads(heads, s0 + base, len, kmax, calls, n_glob, a.ks);
-    __syncwarp();
+  const size_t part_pitch = static_cast<size_t>(a.geo.S) * t.tiles * NOCC;  // entries of one record
+  ScaPart* part = t.parts + (static_cast<size_t>(sample) * t.tiles + tile) * NOCC;
+  const uint64_t* next_time = a.times + a.clock->next_time + t.rec_offset;
+  uint32_t filled = 0, base = 0, recs = 0;
+  for (uint32_t done = 0; done < t.n;) {
+    if (done == filled) {
+      base = done;
+      filled = min(done + chunk, t.n);
+      __syncwarp();
+      sca_fill_heads(heads, s0 + base, filled - base, kmax, calls, n_glob, a.ks);
+      __syncwarp();
+    }
+    uint32_t stop = filled;
+    if (recs < t.n_rec) stop = static_cast<uint32_t>(min(static_cast<uint64_t>(stop), next_time[recs] - s0));
 #pragma unroll 1
-    for (uint32_t it = 0; it < len; ++it) {
+    for (; done < stop; ++done) {
+      const uint32_t it = done - base;
       const uint4* hd = heads.head + it * calls;
       const uint32_t a0 = heads.a0[it];
       uint32_t h[UPT][4];
@@ -204,7 +296,13 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
                        : sca_turn_pool<1>(U[0][0], U[NOCC - 1][0], Q[0], *turn, gu[0], counted[0], a0, b2,
                                           hd[kmax + 1], a);
     }
+    if (recs < t.n_rec && next_time[recs] == s0 + done) {
+      tile_record<NOCC, UPT>(U, gu, counted, a, sample, s0 + done, part, COUNT, cnt);
+      part += part_pitch;
+      ++recs;
+    }
   }
+  if (COUNT && t.n_rec) tile_hops(cnt, part);
 
 #pragma unroll
   for (uint32_t j = 0; j < UPT; ++j) {
@@ -228,6 +326,74 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
       for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
       if (lane == 0u && v) atomicAdd(reinterpret_cast<unsigned long long*>(a.counters + 4ull * sample + k), v);
     }
+  }
+}
+
+// The records of one launch, a warp per record and sample: the tiles' sums
+// with their entry heights H_j added back exactly (sum (H + h') = sum h' + H n,
+// sum (H + h')^2 = sum h'^2 + 2 H sum h' + H^2 n), and the hop counters at the
+// record: those after the launch, less the launch's hops, plus its hops so far.
+__global__ void __launch_bounds__(128) k_sca_records(const DomainLaunch a, const ScaTileLaunch t) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint64_t item = static_cast<uint64_t>(blockIdx.x) * 4u + (threadIdx.x >> 5);
+  const uint32_t S = a.geo.S, planes = a.geo.planes, n_units = a.geo.W / 8u;
+  if (item >= static_cast<uint64_t>(t.n_rec) * S) return;  // whole warps
+  const uint32_t r = static_cast<uint32_t>(item / S), sample = static_cast<uint32_t>(item - static_cast<uint64_t>(r) * S);
+  const size_t slot = static_cast<size_t>(a.clock->next_time) + t.rec_offset + r;
+  const ScaPart* mine = t.parts + (static_cast<size_t>(r) * S + sample) * t.tiles * planes;
+  const ScaPart* after = t.parts + (static_cast<size_t>(t.n_rec) * S + sample) * t.tiles * planes;
+  long long hops[4] = {0, 0, 0, 0};
+  for (uint32_t p = 0; p < planes; ++p) {
+    long long H = 0, s1 = 0, ov = 0;
+    __int128 s2 = 0;
+    for (uint32_t j0 = 0; j0 < t.tiles; j0 += 32u) {
+      const uint32_t j = j0 + lane;
+      const bool in = j < t.tiles;
+      ScaPart q = {};
+      if (in) {
+        q = mine[static_cast<size_t>(j) * planes + p];
+        if (p == 0 && a.count_hops) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            hops[k] += static_cast<long long>(q.hops[k]) - after[static_cast<size_t>(j) * planes].hops[k];
+        }
+      }
+      long long incl = q.tot;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const long long v = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= static_cast<uint32_t>(d)) incl += v;
+      }
+      const long long h = H + incl - q.tot, n = in ? 256ll * min(t.units, n_units - j * t.units) : 0ll;
+      s1 += q.s1 + h * n;
+      s2 += static_cast<__int128>(q.s2) + static_cast<__int128>(2 * h) * q.s1 + static_cast<__int128>(h) * h * n;
+      ov += q.ov;
+      H += __shfl_sync(0xffffffffu, incl, 31);
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      s1 += __shfl_xor_sync(0xffffffffu, s1, d);
+      ov += __shfl_xor_sync(0xffffffffu, ov, d);
+      const unsigned long long lo = __shfl_xor_sync(0xffffffffu, static_cast<unsigned long long>(s2), d);
+      const unsigned long long hi =
+          __shfl_xor_sync(0xffffffffu, static_cast<unsigned long long>(static_cast<unsigned __int128>(s2) >> 64), d);
+      s2 += static_cast<__int128>((static_cast<unsigned __int128>(hi) << 64) | lo);
+    }
+    if (lane == 0u) {
+      const size_t e = (slot * S + sample) * planes + p;
+      a.tab_sh[e] = s1;
+      a.tab_sh2[2 * e] = static_cast<uint64_t>(static_cast<unsigned __int128>(s2));
+      a.tab_sh2[2 * e + 1] = static_cast<uint64_t>(static_cast<unsigned __int128>(s2) >> 64);
+      if (a.ex.snap) a.ex.tab_ac[e] = ov;
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) hops[k] += __shfl_xor_sync(0xffffffffu, hops[k], d);
+    if (lane == 0u)
+      a.ex.tab_cnt[(slot * S + sample) * 4 + k] =
+          static_cast<int64_t>(a.counters[4ull * sample + k]) + hops[k];
   }
 }
 
@@ -323,15 +489,26 @@ size_t sca_halo_words(const ScaTiles& t, uint32_t S, uint32_t planes) {
   return static_cast<size_t>(2u) * S * t.tiles * 2u * planes * 8u;
 }
 
-cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, uint32_t* halo, bool fresh, uint32_t* parity,
-                       uint32_t* launches, cudaStream_t st) {
+uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t tiles, uint32_t planes) {
+  uint32_t most = 0;  // sample times in any kScaTileSweeps consecutive sweeps
+  for (size_t i = 0, j = 0; j < n; ++j) {
+    while (times[j] - times[i] >= kScaTileSweeps) ++i;
+    most = std::max(most, static_cast<uint32_t>(j - i + 1));
+  }
+  // no more than 64 MB or a record's worth
+  const uint64_t one = static_cast<uint64_t>(S) * tiles * planes * sizeof(ScaPart);
+  return static_cast<uint32_t>(std::min<uint64_t>(most, std::max<uint64_t>(1u, (64ull << 20) / one)));
+}
+
+cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, const ScaRun& run, cudaStream_t st,
+                       uint32_t* launches) {
   const size_t half = sca_halo_words(tiles, a.geo.S, a.geo.planes) / 2u;
-  if (!fresh) {
+  uint32_t parity = 0, rec = 0;
+  {
     (void)cudaGetLastError();
     const size_t n16 = half / 4u;
     const uint32_t blocks = static_cast<uint32_t>(std::min<size_t>((n16 + 255u) / 256u, 152u * 16u));
-    k_sca_halo<<<blocks, 256, 0, st>>>(a.state, halo + *parity * half, a.geo.S, a.geo.planes, a.geo.W, tiles.tiles,
-                                       tiles.units);
+    k_sca_halo<<<blocks, 256, 0, st>>>(a.state, run.halo, a.geo.S, a.geo.planes, a.geo.W, tiles.tiles, tiles.units);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
     ++*launches;
@@ -340,15 +517,32 @@ cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, uint32_t* h
     ScaTileLaunch t;
     t.tiles = tiles.tiles;
     t.units = tiles.units;
-    t.n = std::min(kScaTileSweeps, a.n_sweeps - done);
+    t.n = std::min({kScaTileSweeps, run.max_sweeps, a.n_sweeps - done});
     t.offset = done;
-    t.halo_in = halo + *parity * half;
-    t.halo_out = halo + (*parity ^ 1u) * half;
-    const cudaError_t e = launch_tiles(a, t, tiles.upt, st);
+    t.rec_offset = rec;
+    t.n_rec = 0;
+    while (rec + t.n_rec < run.n_times && run.times[rec + t.n_rec] - run.sweep <= done + t.n) {
+      if (t.n_rec == run.max_records) {  // the launch ends before the first record it has no room for
+        t.n = static_cast<uint32_t>(run.times[rec + t.n_rec - 1] - run.sweep) - done;
+        break;
+      }
+      ++t.n_rec;
+    }
+    t.halo_in = run.halo + parity * half;
+    t.halo_out = run.halo + (parity ^ 1u) * half;
+    t.parts = run.parts;
+    cudaError_t e = launch_tiles(a, t, tiles.upt, st);
     if (e != cudaSuccess) return e;
-    *parity ^= 1u;
-    done += t.n;
     ++*launches;
+    if (t.n_rec) {
+      const uint64_t items = static_cast<uint64_t>(t.n_rec) * a.geo.S;
+      k_sca_records<<<static_cast<uint32_t>((items + 3u) / 4u), 128, 0, st>>>(a, t);
+      if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      ++*launches;
+    }
+    parity ^= 1u;
+    rec += t.n_rec;
+    done += t.n;
   }
   return cudaSuccess;
 }
