@@ -536,6 +536,9 @@ DomainLaunch domain_desc(const asep_ctx* ctx, uint32_t n) {
     // every warp inside one sample, and the idle realign buffer holds 5 words per column
     const uint32_t np = (ctx->p.model == ASEP_MODEL_TWO_LANE ? 2u : 1u) + dis_planes(ctx->p.dis_kind);
     a.lane_sort = (ctx->cluster <= 1 && ctx->G % 32 == 0 && np * (ctx->R2 + 1) >= 5) ? 1u : 0u;
+    // ... and, behind them, a table of four words per call for each of its samples
+    const uint32_t calls = (a.ptab_klo + a.ptab_n) / 4u + 3u;
+    a.heads = a.lane_sort && 4ull * calls * ctx->spc <= (np * (ctx->R2 + 1ull) - 5u) * ctx->Cp ? calls : 0u;
   }
   a.rates = rates(ctx);
   {

@@ -25,6 +25,33 @@ __device__ __forceinline__ uint32_t poisson_count(const uint32_t* tab, uint32_t 
   return klo + lo;
 }
 
+// The attempts' accesses to shared memory, by 32-bit address.  They keep their
+// order among themselves; attempts_fence keeps the ordinary accesses before
+// and after a phase's attempts on their sides.
+// The stores of a hop are predicated explicitly: as a C++ condition they
+// became a branch around them, which ended the basic block at every attempt,
+// so nothing of the next Philox call could run in the shadow of an attempt's
+// load, test and store.  us per sweep with the branch and without: 8 rings of
+// 4096 41.0 -> 32.2, 256 rings of 2^16 with bimodal disorder 53.9 -> 44.4, 128
+// pairs of lanes of 2^16 51.7 -> 47.3, 256 rings of 2^17 52.4 -> 47.0, 16
+// streamed rings of 2^24 431 -> 415 (all with the shared rounds below, which
+// alone gave 1 % at most).
+__device__ __forceinline__ void attempts_fence() { asm volatile("" ::: "memory"); }
+__device__ __forceinline__ uint32_t lds(uint32_t addr) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ void sts_if(bool p, uint32_t addr0, uint32_t v0, uint32_t addr1, uint32_t v1) {
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "setp.ne.u32 p, %4, 0;\n"
+      "@p st.shared.u32 [%0], %1;\n"
+      "@p st.shared.u32 [%2], %3;\n"
+      "}\n" ::"r"(addr0), "r"(v0), "r"(addr1), "r"(v1), "r"(static_cast<uint32_t>(p)));
+}
+
 struct Cnt {
   uint32_t a = 0, b = 0, c = 0, d = 0;  // ring: right, left; two lanes: A hops, B hops, A->B, B->A
 };
@@ -40,7 +67,8 @@ struct Lane {
   bool active;
 };
 
-// One attempt of a half-domain phase, without branches.  The bond's two
+// One attempt of a half-domain phase, without branches (cur: 32-bit shared
+// address of the columns).  The bond's two
 // words are rows `row` and `row + 1` of the lane's own column (row 2D/32 is
 // the mirror of the next column's row 0), both loaded unconditionally; the
 // 64-bit flip mask (3 << j across the word pair) is applied under one
@@ -56,7 +84,7 @@ struct Lane {
 // the test equals u < t of the definition; the other two patterns fall
 // outside the window.
 template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP>
-__device__ __forceinline__ void attempt(unsigned char* cur, const DomainLaunch& a, uint32_t PWb, uint32_t base_b,
+__device__ __forceinline__ void attempt(uint32_t cur, const DomainLaunch& a, uint32_t PWb, uint32_t base_b,
                                         uint32_t row_scale_b, uint32_t r, bool valid, Cnt& cnt) {
   // byte offset of row (j >> 5) of this half: (r & (D - 1) & ~31) * (4 Cp / 32)
   const uint32_t cpb = CP ? CP * 4u : a.Cp * 4u;  // row pitch in bytes (compile-time when CP != 0)
@@ -67,22 +95,21 @@ __device__ __forceinline__ void attempt(unsigned char* cur, const DomainLaunch& 
     laneB = (r >> a.logD) & 1u;  // lane A hops right only (p), lane B left only (q)
     o0 += laneB * PWb;
   } else if (DIS == kDisBimodal || DIS == kDisBimodalPQ) {
-    const uint32_t c0 = *reinterpret_cast<const uint32_t*>(cur + PWb + o0);
-    const uint32_t c1 = *reinterpret_cast<const uint32_t*>(cur + PWb + o0 + cpb);
+    const uint32_t c0 = lds(cur + PWb + o0);
+    const uint32_t c1 = lds(cur + PWb + o0 + cpb);
     const uint32_t pc = __funnelshift_r(c0, c1, r);  // bit0: class of site i, bit1: of site i+1
     uint32_t qc = pc;
     if (DIS == kDisBimodalPQ) {  // left hops take the class of site i+1 from the second quenched plane
-      const uint32_t d0 = *reinterpret_cast<const uint32_t*>(cur + 2u * PWb + o0);
-      const uint32_t d1 = *reinterpret_cast<const uint32_t*>(cur + 2u * PWb + o0 + cpb);
+      const uint32_t d0 = lds(cur + 2u * PWb + o0);
+      const uint32_t d1 = lds(cur + 2u * PWb + o0 + cpb);
       qc = __funnelshift_r(d0, d1, r);
     }
     bR = (pc & 1u) ? a.rates.pb_slow : bR;  // right hop across (i, i+1): p_i
     bL = (qc & 2u) ? a.rates.qb_slow : bL;  // left hop: q_{i+1}
   }
-  uint32_t* p0 = reinterpret_cast<uint32_t*>(cur + o0);
-  uint32_t* p1 = reinterpret_cast<uint32_t*>(cur + o0 + cpb);
-  const uint32_t w0 = *p0;
-  const uint32_t w1 = *p1;
+  const uint32_t p0 = cur + o0, p1 = cur + o0 + cpb;
+  const uint32_t w0 = lds(p0);
+  const uint32_t w1 = lds(p1);
   const uint32_t key = __funnelshift_l(r, __funnelshift_r(w0, w1, r), 30);
   bool hopL = static_cast<int32_t>(key) < bL;
   bool hopR = static_cast<int32_t>(key + 0x40000000u) < bR;
@@ -90,13 +117,94 @@ __device__ __forceinline__ void attempt(unsigned char* cur, const DomainLaunch& 
     hopR = hopR && !laneB;
     hopL = hopL && laneB;
   }
-  if (valid && (hopR || hopL)) {
-    *p0 = w0 ^ __funnelshift_l(0u, 3u, r);  // 3 << (j mod 32), truncated
-    *p1 = w1 ^ __funnelshift_l(3u, 0u, r);  // 1 when j mod 32 == 31, else 0
-  }
+  sts_if(valid && (hopR || hopL), p0, w0 ^ __funnelshift_l(0u, 3u, r),  // 3 << (j mod 32), truncated
+         p1, w1 ^ __funnelshift_l(3u, 0u, r));                          // 1 when j mod 32 == 31, else 0
   if (COUNT) {
     cnt.a += valid && hopR;
     cnt.b += valid && hopL;
+  }
+}
+
+// The draws of one domain at one sweep: call c of the attempt stream (tag DOM,
+// counter (s, tag | c << 12, sample, domain)) with the rounds that lanes or
+// calls share taken out (asep_device.cuh).  With a table of heads (one entry
+// per call, shared by all domains of the sample and both phases) a call costs
+// a lane 14 wide multiplies and one broadcast load, without one 16, instead of
+// 20.
+template <bool TABLE>
+struct DomainStream {
+  const uint4* heads;  // shared memory, entry c = call c (TABLE); else the head of every call is formed
+  PhiloxLane lane;
+  uint32_t h1, e1;     // without a table: round 1 of word 2 (without the call), round 2's XOR of word 2
+
+  // table: whether the heads come from `h`; s: sweep; n: sample id; d: domain.
+  __device__ __forceinline__ void open(const uint4* h, uint64_t s, uint32_t n, uint32_t d, const KeySchedule& ks) {
+    const uint2 p0 = mul_wide(0xD2511F53u, static_cast<uint32_t>(s)), p1 = mul_wide(0xCD9E8D57u, n);
+    heads = h;
+    lane = philox_lane(p0.y ^ ks.y[0], p1.x ^ ks.x[1], d);
+    h1 = p1.y ^ ks.x[0] ^ ctr_of(s, kTagDom, 0, 0, 0).y;
+    e1 = p0.x ^ ks.y[1];
+  }
+  __device__ __forceinline__ uint4 draw(uint32_t call, const KeySchedule& ks) const {
+    PhiloxHead h;
+    if (TABLE) {
+      const uint4 v = heads[call];
+      h = PhiloxHead{v.x, v.y, v.z};
+    } else {
+      const uint2 q = mul_wide(0xD2511F53u, h1 ^ (call << 12));
+      const uint2 r = mul_wide(0xCD9E8D57u, q.y ^ e1);
+      h = PhiloxHead{r.y ^ ks.x[2], r.x, q.x ^ ks.y[2]};
+    }
+    return philox_tail(h, lane, ks);
+  }
+};
+
+// Entries of a sample's table of heads: every call of the largest count, and
+// the one drawn ahead of it.
+__host__ __device__ inline uint32_t domain_calls(uint32_t ptab_klo, uint32_t ptab_n) { return (ptab_klo + ptab_n) / 4u + 3u; }
+
+// Entry `call` of the table of sample id n at sweep s.
+__device__ __forceinline__ uint4 domain_head(uint64_t s, uint32_t call, uint32_t n, const KeySchedule& ks) {
+  const PhiloxHead h = philox_head(static_cast<uint32_t>(s), ctr_of(s, kTagDom, call, 0, 0).y, n, ks);
+  return make_uint4(h.c3, h.y3, h.d3, 0u);
+}
+
+// Calls whose four attempts every lane of the warp makes (k + 3 <= Kmin) need
+// no per-attempt count test; the remaining calls up to Kmax test k <= K.  A
+// domain's attempts keep their order either way.  The fast calls are
+// 1 .. (Kmin - 3) / 4.  Each iteration draws the next call's words before it
+// applies the current call's four attempts (the random stream does not
+// depend on the lattice), so Philox's rounds overlap the attempts' dependent
+// chain; two iterations per loop trip.
+template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP, bool TABLE>
+__device__ __forceinline__ void run_calls(uint32_t cb, const uint4* heads, const DomainLaunch& a, uint32_t PWb,
+                                          uint32_t base_b, uint32_t row_scale_b, uint64_t s, uint32_t n_glob,
+                                          uint32_t dd, uint32_t K, uint32_t Kmin, uint32_t Kmax, Cnt& cnt) {
+  DomainStream<TABLE> ds;
+  ds.open(heads, s, n_glob, dd, a.ks);
+  const uint32_t n_fast = Kmin >= 3u ? (Kmin - 3u) >> 2 : 0u;
+  uint32_t call = 1;
+  uint4 y = ds.draw(1, a.ks);  // call n_fast + 1's words when the fast loop ends
+#pragma unroll 2
+  for (; call <= n_fast;) {
+    ++call;
+    const uint4 yn = ds.draw(call, a.ks);  // the next call, ahead of this call's attempts
+    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.x, true, cnt);
+    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.y, true, cnt);
+    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.z, true, cnt);
+    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.w, true, cnt);
+    y = yn;
+  }
+#pragma unroll 1
+  for (; (call << 2) <= Kmax; ++call) {
+    const uint32_t k = call << 2;
+    uint4 yn = y;
+    if (k + 4 <= Kmax) yn = ds.draw(call + 1, a.ks);  // warp-uniform
+    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.x, k <= K, cnt);
+    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.y, k + 1 <= K, cnt);
+    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.z, k + 2 <= K, cnt);
+    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.w, k + 3 <= K, cnt);
+    y = yn;
   }
 }
 
@@ -113,15 +221,21 @@ __device__ __forceinline__ void attempt(unsigned char* cur, const DomainLaunch& 
 // shrink.  `scr` is the idle realign buffer (overwritten by the next realign).
 // The cluster tier passes sort = false: there other CTAs may still read that
 // buffer remotely during the first phase.
-template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP, uint32_t PHASE>
-__device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sort, const DomainLaunch& a,
-                                          const uint32_t* tab, uint32_t PW, uint64_t s, const Lane& ln, uint2 key,
-                                          Cnt& cnt) {
+//
+// heads: the sample's table of heads, or nullptr.  fill: the table is formed
+// here, between the two barriers of the lane sort (the first phase of a
+// sweep), in the idle buffer behind the sort's scratch.
+template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP, uint32_t PHASE, bool TABLE>
+__device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sort, uint4* heads, bool fill,
+                                          const DomainLaunch& a, const uint32_t* tab, uint32_t PW, uint64_t s,
+                                          const Lane& ln, Cnt& cnt) {
   const uint32_t d = 2 * ln.g + PHASE;
   uint4 x0 = make_uint4(0u, 0u, 0u, 0u);
   uint32_t K = 0;
+  DomainStream<false> ds;
   if (ln.active) {
-    x0 = philox10(ctr_of(s, kTagDom, 0, ln.n_glob, d), a.ks);
+    ds.open(nullptr, s, ln.n_glob, d, a.ks);
+    x0 = ds.draw(0, a.ks);
     K = poisson_count(tab, a.ptab_n, a.ptab_klo, x0.x);
   }
   const uint32_t cp = CP ? CP : a.Cp;
@@ -139,6 +253,10 @@ __device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sor
       sX[ln.c] = x0.y;
       sX[cp + ln.c] = x0.z;
       sX[2 * cp + ln.c] = x0.w;
+      if (fill) {  // the sample's threads share the entries out
+        const uint32_t calls = domain_calls(a.ptab_klo, a.ptab_n);
+        for (uint32_t c = ln.g; c < calls; c += a.G) heads[c] = domain_head(s, c, ln.n_glob, a.ks);
+      }
     }
     __syncthreads();
     if (in_group) {
@@ -162,49 +280,19 @@ __device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sor
   }
   const uint32_t Kmax = __reduce_max_sync(0xffffffffu, K);
   const uint32_t Kmin = __reduce_min_sync(0xffffffffu, K);
-  unsigned char* cb = reinterpret_cast<unsigned char*>(cur);
+  const uint32_t cb = static_cast<uint32_t>(__cvta_generic_to_shared(cur));
   const uint32_t base_b = (PHASE * (a.D >> 5) * cp + col) * 4u;
   const uint32_t row_scale_b = cp >> 3;  // 4 * Cp / 32
   const uint32_t PWb = PW * 4u;
+  attempts_fence();
   attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, x0.y, 1 <= K, cnt);
   attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, x0.z, 2 <= K, cnt);
   attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, x0.w, 3 <= K, cnt);
-  // Calls whose four attempts every lane of the warp makes (k + 3 <= Kmin) need
-  // no per-attempt count test; the remaining calls up to Kmax test k <= K.  A
-  // domain's attempts keep their order either way.  The fast calls are
-  // 1 .. (Kmin - 3) / 4; call k's counter is call 1's with k - 1 added at bit 12
-  // of word 1 (the call field), so the loop steps that word.  Each iteration
-  // draws the next call's words before it applies the current call's four
-  // attempts (the random stream does not depend on the lattice), so Philox's
-  // rounds overlap the attempts' dependent chain; two iterations per loop trip.
-  uint4 ctr = ctr_of(s, kTagDom, 1, ln.n_glob, dd);
-  const uint32_t n_fast = Kmin >= 3u ? (Kmin - 3u) >> 2 : 0u;
-  const uint32_t y_end = ctr.y + (n_fast << 12);
-  uint4 y = philox10(ctr, a.ks);  // call n_fast + 1's words when the fast loop ends
-#pragma unroll 2
-  for (; ctr.y != y_end;) {
-    ctr.y += 1u << 12;
-    const uint4 yn = philox10(ctr, a.ks);  // the next call, ahead of this call's attempts
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.x, true, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.y, true, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.z, true, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.w, true, cnt);
-    y = yn;
-  }
-#pragma unroll 1
-  for (uint32_t call = n_fast + 1; (call << 2) <= Kmax; ++call) {
-    const uint32_t k = call << 2;
-    uint4 yn = y;
-    if (k + 4 <= Kmax) {  // warp-uniform
-      ctr.y += 1u << 12;
-      yn = philox10(ctr, a.ks);
-    }
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.x, k <= K, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.y, k + 1 <= K, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.z, k + 2 <= K, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.w, k + 3 <= K, cnt);
-    y = yn;
-  }
+  if (TABLE && heads)
+    run_calls<MODEL, DIS, COUNT, CP, true>(cb, heads, a, PWb, base_b, row_scale_b, s, ln.n_glob, dd, K, Kmin, Kmax, cnt);
+  else
+    run_calls<MODEL, DIS, COUNT, CP, false>(cb, heads, a, PWb, base_b, row_scale_b, s, ln.n_glob, dd, K, Kmin, Kmax, cnt);
+  attempts_fence();
 }
 
 }  // namespace

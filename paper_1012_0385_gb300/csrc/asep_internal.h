@@ -114,6 +114,7 @@ struct DomainLaunch {
   uint32_t cluster;        // CTAs per sample: 1 = resident in one CTA, 2..16 = a thread-block cluster
   uint32_t Gc;             // cluster tier: columns per CTA (the last CTA may hold fewer)
   uint32_t lane_sort;      // resident tier: warps run domains of similar Poisson count (results unchanged)
+  uint32_t heads;          // resident tier with the lane sort: entries of a sample's table of heads (0 = no table)
   uint32_t sca_kmax;       // SCA: random planes that decide every threshold (20 - fewest trailing zeros)
   Rates rates;
   uint64_t seed;

@@ -493,14 +493,14 @@ __global__ void __launch_bounds__(1024) k_cluster(const DomainLaunch a) {
     nxt = t;
     R_cur = o;
     __syncthreads();
-    run_phase<MODEL, DIS, COUNT, 0, 0>(cur, nullptr, false, a, tab, PW, s, ln, key, cnt);
+    run_phase<MODEL, DIS, COUNT, 0, 0, false>(cur, nullptr, false, nullptr, false, a, tab, PW, s, ln, cnt);
     cl.sync();
     if (ln.active) {
 #pragma unroll
       for (uint32_t p = 0; p < NP; ++p)
         cur[p * PW + R2 * Cp + ln.c] = *cl_word(cl, cur, p, PW, 0, Cp, gn, Gc, my_rank);
     }
-    run_phase<MODEL, DIS, COUNT, 0, 1>(cur, nullptr, false, a, tab, PW, s, ln, key, cnt);
+    run_phase<MODEL, DIS, COUNT, 0, 1, false>(cur, nullptr, false, nullptr, false, a, tab, PW, s, ln, cnt);
     cl.sync();
     if (ln.active) {
 #pragma unroll

@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(1024) k_stream(const DomainLaunch a, uint32_t 
   ln.n_glob = n_glob;
   ln.active = c < Cn;
   Cnt cnt;
-  run_phase<MODEL, DIS, COUNT, 0, PHASE>(cols, nullptr, false, a, tab, PW, s, ln, key, cnt);
+  run_phase<MODEL, DIS, COUNT, 0, PHASE, false>(cols, nullptr, false, nullptr, false, a, tab, PW, s, ln, cnt);
   __syncthreads();
   if (PHASE == 1) {  // the last bond of column c reached row 0 of column c + 1 through its mirror row
     if (c + 1 < Cn) {
