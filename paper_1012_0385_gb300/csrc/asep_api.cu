@@ -59,6 +59,7 @@ struct asep_ctx {
   uint32_t R2 = 0, logR2 = 0, G = 0, spc = 1, C = 0, Cp = 0, threads = 0, blocks = 0;
   uint32_t cluster = 1, Gc = 0;  // cluster tier: CTAs per sample, columns per CTA (kStreamTier: streamed)
   uint32_t tiles = 0;             // streamed tier: tiles per sample
+  uint32_t heads_at = 0;          // cluster and streamed tiers: offset of the table of heads in shared memory (0 = none)
   uint32_t* d_err = nullptr;      // device flag: a streamed tile's copy wait gave up
   uint32_t fault = ASEP_FAULT_NONE;  // injected fault (asep_inject_fault)
   size_t smem = 0;
@@ -324,6 +325,7 @@ int plan_domain(asep_ctx* ctx, uint32_t force_cluster, uint32_t force_spc) {
   ctx->G = static_cast<uint32_t>(G);
   const uint32_t dis = ctx->p.dis_kind;
   const uint32_t ptab_n = static_cast<uint32_t>(ctx->ptab.size());
+  const uint32_t calls = domain_calls(ctx->ptab_klo, ptab_n);
   bool placed = false;
   if (G <= 1024 && force_cluster <= 1) {
     uint32_t spc = force_spc ? force_spc : 1;
@@ -333,6 +335,7 @@ int plan_domain(asep_ctx* ctx, uint32_t force_cluster, uint32_t force_spc) {
       const uint32_t Cp = (C + 31) / 32 * 32;
       const size_t smem = domain_smem_bytes(ctx->p.model, dis, ctx->R2, Cp, ptab_n, Cp);
       if (smem <= 227 * 1024 && Cp <= 1024) {
+        ctx->heads_at = 0;  // the resident tier keeps it in the idle buffer
         ctx->cluster = 1;
         ctx->Gc = 0;
         ctx->spc = spc;
@@ -357,13 +360,17 @@ int plan_domain(asep_ctx* ctx, uint32_t force_cluster, uint32_t force_spc) {
     const uint32_t Cp = (Gc + 31) / 32 * 32;
     const size_t smem = domain_smem_bytes(ctx->p.model, dis, ctx->R2, Cp, ptab_n, Cp);
     if (ok && smem + 64 <= 227 * 1024 && Cp <= 1024 && cluster_fits(ctx->p.model, dis, nc, Cp, smem) > 0) {
+      // the table of random heads behind the rest, where that still fits
+      const size_t at = (smem + 15) & ~static_cast<size_t>(15), with = at + 16ull * calls;
+      const bool table = with + 64 <= 227 * 1024 && cluster_fits(ctx->p.model, dis, nc, Cp, with) > 0;
+      ctx->heads_at = table ? static_cast<uint32_t>(at) : 0u;
       ctx->cluster = nc;
       ctx->spc = 1;
       ctx->C = Gc;
       ctx->Gc = Gc;
       ctx->Cp = Cp;
       ctx->threads = Cp;
-      ctx->smem = smem;
+      ctx->smem = table ? with : smem;
       ctx->blocks = ctx->S;
       placed = true;
     }
@@ -385,7 +392,8 @@ int plan_domain(asep_ctx* ctx, uint32_t force_cluster, uint32_t force_spc) {
       ctx->Gc = 0;
       ctx->Cp = C;
       ctx->threads = C;
-      ctx->smem = smem;
+      ctx->heads_at = static_cast<uint32_t>((smem + 15) & ~static_cast<size_t>(15));
+      ctx->smem = ctx->heads_at + 16ull * calls;  // at most 200 KB + 17 KB (D = 2048)
       ctx->tiles = static_cast<uint32_t>((G + C - 1) / C);
       ctx->blocks = ctx->tiles * ctx->S;
       placed = true;
@@ -536,11 +544,15 @@ DomainLaunch domain_desc(const asep_ctx* ctx, uint32_t n) {
     // every warp inside one sample, and the idle realign buffer holds 5 words per column
     const uint32_t np = (ctx->p.model == ASEP_MODEL_TWO_LANE ? 2u : 1u) + dis_planes(ctx->p.dis_kind);
     a.lane_sort = (ctx->cluster <= 1 && ctx->G % 32 == 0 && np * (ctx->R2 + 1) >= 5) ? 1u : 0u;
-    // ... and, behind them, a table of four words per call for each of its samples
-    const uint32_t calls = (a.ptab_klo + a.ptab_n) / 4u + 3u;
-    a.heads = a.lane_sort && 4ull * calls * ctx->spc <= (np * (ctx->R2 + 1ull) - 5u) * ctx->Cp ? calls : 0u;
+    // ... and, behind them, a table of four words per call for each of its samples (from some 25 columns on)
+    const uint32_t calls = domain_calls(a.ptab_klo, a.ptab_n);
+    const bool fits = 4ull * calls * ctx->spc <= (np * (ctx->R2 + 1ull) - (a.lane_sort ? 5u : 0u)) * ctx->Cp;
+    a.heads = ctx->cluster <= 1 ? (fits ? calls : 0u) : (ctx->heads_at ? calls : 0u);
+    a.heads_at = ctx->heads_at;
   }
   a.rates = rates(ctx);
+  a.left = ctx->p.model == ASEP_MODEL_RING && (a.rates.q || a.rates.q_slow) ? 1u : 0u;
+  a.inverse = a.left ? 0u : ~0u;
   {
     // SCA: planes needed to decide u < t for every threshold that is neither 0 nor always
     uint32_t tz = 20;
@@ -1485,6 +1497,7 @@ int asep_set_plan(asep_ctx* ctx, uint32_t cluster, uint32_t samples_per_group) {
     ctx->smem = saved.smem;
     ctx->blocks = saved.blocks;
     ctx->tiles = saved.tiles;
+    ctx->heads_at = saved.heads_at;
     ctx->max_sweeps_per_launch = saved.max_sweeps_per_launch;
     ctx->err = msg;
   }

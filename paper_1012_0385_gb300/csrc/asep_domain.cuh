@@ -56,6 +56,15 @@ struct Cnt {
   uint32_t a = 0, b = 0, c = 0, d = 0;  // ring: right, left; two lanes: A hops, B hops, A->B, B->A
 };
 
+template <bool B>
+struct Flag {
+  static constexpr bool value = B;
+};
+
+// Plane p of the columns holds the sites' complement where this is all ones
+// (see attempt).
+__device__ __forceinline__ uint32_t plane_inverse(const DomainLaunch& a, uint32_t p) { return p == 0 ? a.inverse : 0u; }
+
 struct Lane {
   uint32_t c;        // column in the CTA
   uint32_t g;        // super-domain index within the sample
@@ -67,61 +76,73 @@ struct Lane {
   bool active;
 };
 
-// One attempt of a half-domain phase, without branches (cur: 32-bit shared
-// address of the columns).  The bond's two
-// words are rows `row` and `row + 1` of the lane's own column (row 2D/32 is
-// the mirror of the next column's row 0), both loaded unconditionally; the
-// 64-bit flip mask (3 << j across the word pair) is applied under one
-// predicate.  `valid` is k <= K.
+// One attempt of a half-domain phase, without branches (base: 32-bit shared
+// address of the lane's column in the half's first row).  The bond's two words
+// are rows `row` and `row + 1` of the column (row 2D/32 is the mirror of the
+// next column's row 0), both loaded unconditionally; the 64-bit flip mask
+// (3 << j across the word pair) is applied under one predicate.  `valid` is
+// k <= K.
 //
-// Both hop tests come from one key: bits 31 and 30 hold sites i+1 and i (the
-// funnel-shifted word pair), bits 29..0 hold r >> 2.  A left hop (sites 01,
-// key bits 10) is accepted iff the key, read as signed, lies below
-// INT_MIN + t/4 for the left rate t; adding 2^30 carries a right-hop pattern
-// (bits 01) into the same window, tested against the right rate's bound
+// The hop test takes one key: bits 31 and 30 hold sites i+1 and i (the
+// funnel-shifted word pair), bits 29..0 hold r >> 2.  Sites 01 (key bits 10)
+// are accepted iff the key, read as signed, lies below INT_MIN + t/4
 // (hop_bound: INT_MIN + t/4, INT_MIN + 2^30 for "always", INT_MIN for 0).
 // Thresholds are multiples of 4096, for which r < t iff r >> 2 < t >> 2, so
-// the test equals u < t of the definition; the other two patterns fall
-// outside the window.
-template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP>
-__device__ __forceinline__ void attempt(uint32_t cur, const DomainLaunch& a, uint32_t PWb, uint32_t base_b,
-                                        uint32_t row_scale_b, uint32_t r, bool valid, Cnt& cnt) {
-  // byte offset of row (j >> 5) of this half: (r & (D - 1) & ~31) * (4 Cp / 32)
+// the test equals u < t of the definition; the other patterns fall outside
+// the window.  Pattern 10 is brought into it by adding 2^30 to the key or,
+// where every hop of a plane goes the same way, by keeping the plane's
+// complement in shared memory: lane A of two lanes, and rings without left
+// hops (LEFT = false), so that one compare does (plane_inverse).  us per sweep
+// before and after: 8 rings of 4096 at q = 0 32.2 -> 26.5, 256 bimodal rings of
+// 2^16 44.4 -> 36.4 (one class word instead of two, no selects), 128 pairs of
+// lanes of 2^16 47.3 -> 41.8 (with the pooled lane changes).
+//   left hops:  sites 01, bound of q_{i+1};   right hops: sites 10, p_i.
+template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP, bool LEFT>
+__device__ __forceinline__ void attempt(uint32_t base, const DomainLaunch& a, uint32_t PWb, uint32_t row_scale_b,
+                                        uint32_t r, bool valid, Cnt& cnt) {
   const uint32_t cpb = CP ? CP * 4u : a.Cp * 4u;  // row pitch in bytes (compile-time when CP != 0)
-  uint32_t o0 = base_b + (r & a.row_bits) * row_scale_b;
-  int32_t bR = a.rates.pb, bL = a.rates.qb;  // bounds of the right and left hop
+  // row (j >> 5) of this half: (r & (D - 1) & ~31) * (4 Cp / 32)
+  uint32_t p0 = base + (r & a.row_bits) * row_scale_b;
+  uint32_t bR = static_cast<uint32_t>(a.rates.pb), bL = static_cast<uint32_t>(a.rates.qb);
   uint32_t laneB = 0;
   if (MODEL == kTwoLane) {
     laneB = (r >> a.logD) & 1u;  // lane A hops right only (p), lane B left only (q)
-    o0 += laneB * PWb;
-  } else if (DIS == kDisBimodal || DIS == kDisBimodalPQ) {
-    const uint32_t c0 = lds(cur + PWb + o0);
-    const uint32_t c1 = lds(cur + PWb + o0 + cpb);
-    const uint32_t pc = __funnelshift_r(c0, c1, r);  // bit0: class of site i, bit1: of site i+1
-    uint32_t qc = pc;
-    if (DIS == kDisBimodalPQ) {  // left hops take the class of site i+1 from the second quenched plane
-      const uint32_t d0 = lds(cur + 2u * PWb + o0);
-      const uint32_t d1 = lds(cur + 2u * PWb + o0 + cpb);
-      qc = __funnelshift_r(d0, d1, r);
-    }
-    bR = (pc & 1u) ? a.rates.pb_slow : bR;  // right hop across (i, i+1): p_i
-    bL = (qc & 2u) ? a.rates.qb_slow : bL;  // left hop: q_{i+1}
+    p0 += laneB * PWb;
+    bR += laneB * (bL - bR);
   }
-  const uint32_t p0 = cur + o0, p1 = cur + o0 + cpb;
+  const uint32_t p1 = p0 + cpb;
+  if (DIS == kDisBimodal || DIS == kDisBimodalPQ) {
+    // the class bits select by multiplication: (slow - fast) is even
+    const uint32_t dR = static_cast<uint32_t>(a.rates.pb_slow) - bR, dL = (static_cast<uint32_t>(a.rates.qb_slow) - bL) >> 1;
+    const uint32_t c0 = lds(p0 + PWb);
+    if (LEFT) {
+      const uint32_t pc = __funnelshift_r(c0, lds(p1 + PWb), r);  // bit 0: class of site i, bit 1: of site i+1
+      uint32_t qc = pc;
+      if (DIS == kDisBimodalPQ)  // left hops take the class of site i+1 from the second quenched plane
+        qc = __funnelshift_r(lds(p0 + 2u * PWb), lds(p1 + 2u * PWb), r);
+      bR += (pc & 1u) * dR;
+      bL += (qc & 2u) * dL;
+    } else {
+      bR += (__funnelshift_r(c0, c0, r) & 1u) * dR;
+    }
+  }
   const uint32_t w0 = lds(p0);
   const uint32_t w1 = lds(p1);
   const uint32_t key = __funnelshift_l(r, __funnelshift_r(w0, w1, r), 30);
-  bool hopL = static_cast<int32_t>(key) < bL;
-  bool hopR = static_cast<int32_t>(key + 0x40000000u) < bR;
-  if (MODEL == kTwoLane) {
-    hopR = hopR && !laneB;
-    hopL = hopL && laneB;
+  bool hop, left = false;
+  if (MODEL == kTwoLane || !LEFT) {
+    hop = static_cast<int32_t>(key) < static_cast<int32_t>(bR);
+  } else {
+    left = static_cast<int32_t>(key) < static_cast<int32_t>(bL);
+    hop = static_cast<int32_t>(key + 0x40000000u) < static_cast<int32_t>(bR) || left;
   }
-  sts_if(valid && (hopR || hopL), p0, w0 ^ __funnelshift_l(0u, 3u, r),  // 3 << (j mod 32), truncated
-         p1, w1 ^ __funnelshift_l(3u, 0u, r));                          // 1 when j mod 32 == 31, else 0
-  if (COUNT) {
-    cnt.a += valid && hopR;
-    cnt.b += valid && hopL;
+  hop = hop && valid;
+  sts_if(hop, p0, w0 ^ __funnelshift_l(0u, 3u, r),  // 3 << (j mod 32), truncated
+         p1, w1 ^ __funnelshift_l(3u, 0u, r));      // 1 when j mod 32 == 31, else 0
+  if (COUNT) {  // a: all hops, b: left hops (lane B)
+    cnt.a += hop;
+    if (MODEL == kTwoLane) cnt.b += hop ? laneB : 0u;
+    else if (LEFT) cnt.b += hop && left;
   }
 }
 
@@ -159,10 +180,6 @@ struct DomainStream {
   }
 };
 
-// Entries of a sample's table of heads: every call of the largest count, and
-// the one drawn ahead of it.
-__host__ __device__ inline uint32_t domain_calls(uint32_t ptab_klo, uint32_t ptab_n) { return (ptab_klo + ptab_n) / 4u + 3u; }
-
 // Entry `call` of the table of sample id n at sweep s.
 __device__ __forceinline__ uint4 domain_head(uint64_t s, uint32_t call, uint32_t n, const KeySchedule& ks) {
   const PhiloxHead h = philox_head(static_cast<uint32_t>(s), ctr_of(s, kTagDom, call, 0, 0).y, n, ks);
@@ -176,10 +193,16 @@ __device__ __forceinline__ uint4 domain_head(uint64_t s, uint32_t call, uint32_t
 // applies the current call's four attempts (the random stream does not
 // depend on the lattice), so Philox's rounds overlap the attempts' dependent
 // chain; two iterations per loop trip.
-template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP, bool TABLE>
-__device__ __forceinline__ void run_calls(uint32_t cb, const uint4* heads, const DomainLaunch& a, uint32_t PWb,
-                                          uint32_t base_b, uint32_t row_scale_b, uint64_t s, uint32_t n_glob,
-                                          uint32_t dd, uint32_t K, uint32_t Kmin, uint32_t Kmax, Cnt& cnt) {
+template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP, bool TABLE, bool LEFT>
+__device__ __forceinline__ void run_calls(uint32_t base, const uint4* heads, const DomainLaunch& a, uint32_t PWb,
+                                          uint32_t row_scale_b, uint64_t s, uint32_t n_glob, uint32_t dd,
+                                          const uint4 x0, uint32_t K, uint32_t Kmin, uint32_t Kmax, Cnt& cnt) {
+  const auto go = [&](uint32_t r, bool valid) {
+    attempt<MODEL, DIS, COUNT, CP, LEFT>(base, a, PWb, row_scale_b, r, valid, cnt);
+  };
+  go(x0.y, 1 <= K);
+  go(x0.z, 2 <= K);
+  go(x0.w, 3 <= K);
   DomainStream<TABLE> ds;
   ds.open(heads, s, n_glob, dd, a.ks);
   const uint32_t n_fast = Kmin >= 3u ? (Kmin - 3u) >> 2 : 0u;
@@ -189,10 +212,10 @@ __device__ __forceinline__ void run_calls(uint32_t cb, const uint4* heads, const
   for (; call <= n_fast;) {
     ++call;
     const uint4 yn = ds.draw(call, a.ks);  // the next call, ahead of this call's attempts
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.x, true, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.y, true, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.z, true, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.w, true, cnt);
+    go(y.x, true);
+    go(y.y, true);
+    go(y.z, true);
+    go(y.w, true);
     y = yn;
   }
 #pragma unroll 1
@@ -200,10 +223,10 @@ __device__ __forceinline__ void run_calls(uint32_t cb, const uint4* heads, const
     const uint32_t k = call << 2;
     uint4 yn = y;
     if (k + 4 <= Kmax) yn = ds.draw(call + 1, a.ks);  // warp-uniform
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.x, k <= K, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.y, k + 1 <= K, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.z, k + 2 <= K, cnt);
-    attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, y.w, k + 3 <= K, cnt);
+    go(y.x, k <= K);
+    go(y.y, k + 1 <= K);
+    go(y.z, k + 2 <= K);
+    go(y.w, k + 3 <= K);
     y = yn;
   }
 }
@@ -223,8 +246,8 @@ __device__ __forceinline__ void run_calls(uint32_t cb, const uint4* heads, const
 // buffer remotely during the first phase.
 //
 // heads: the sample's table of heads, or nullptr.  fill: the table is formed
-// here, between the two barriers of the lane sort (the first phase of a
-// sweep), in the idle buffer behind the sort's scratch.
+// here (the first phase of a sweep), in the idle buffer behind the sort's
+// scratch, by the sample's threads.
 template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP, uint32_t PHASE, bool TABLE>
 __device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sort, uint4* heads, bool fill,
                                           const DomainLaunch& a, const uint32_t* tab, uint32_t PW, uint64_t s,
@@ -238,6 +261,9 @@ __device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sor
     x0 = ds.draw(0, a.ks);
     K = poisson_count(tab, a.ptab_n, a.ptab_klo, x0.x);
   }
+  if (fill && ln.c < a.C)
+    for (uint32_t c = ln.g; c < a.heads; c += a.G) heads[c] = domain_head(s, c, ln.n_glob, a.ks);
+  if (fill && !sort) __syncthreads();
   const uint32_t cp = CP ? CP : a.Cp;
   uint32_t col = ln.c;  // the column (domain pair) this thread runs
   uint32_t dd = d;      // its domain index in the sample
@@ -253,10 +279,6 @@ __device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sor
       sX[ln.c] = x0.y;
       sX[cp + ln.c] = x0.z;
       sX[2 * cp + ln.c] = x0.w;
-      if (fill) {  // the sample's threads share the entries out
-        const uint32_t calls = domain_calls(a.ptab_klo, a.ptab_n);
-        for (uint32_t c = ln.g; c < calls; c += a.G) heads[c] = domain_head(s, c, ln.n_glob, a.ks);
-      }
     }
     __syncthreads();
     if (in_group) {
@@ -280,19 +302,28 @@ __device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sor
   }
   const uint32_t Kmax = __reduce_max_sync(0xffffffffu, K);
   const uint32_t Kmin = __reduce_min_sync(0xffffffffu, K);
-  const uint32_t cb = static_cast<uint32_t>(__cvta_generic_to_shared(cur));
-  const uint32_t base_b = (PHASE * (a.D >> 5) * cp + col) * 4u;
+  if (Kmax == 0u) return;  // a warp without columns
+  const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(cur)) + (PHASE * (a.D >> 5) * cp + col) * 4u;
   const uint32_t row_scale_b = cp >> 3;  // 4 * Cp / 32
   const uint32_t PWb = PW * 4u;
+  Cnt hops;
+  const auto calls = [&](auto table, auto left) {
+    run_calls<MODEL, DIS, COUNT, CP, decltype(table)::value, decltype(left)::value>(
+        base, heads, a, PWb, row_scale_b, s, ln.n_glob, dd, x0, K, Kmin, Kmax, hops);
+  };
+  constexpr bool kLeft = MODEL == kRing;  // both directions on a plane are possible
+  using No = Flag<false>;
   attempts_fence();
-  attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, x0.y, 1 <= K, cnt);
-  attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, x0.z, 2 <= K, cnt);
-  attempt<MODEL, DIS, COUNT, CP>(cb, a, PWb, base_b, row_scale_b, x0.w, 3 <= K, cnt);
-  if (TABLE && heads)
-    run_calls<MODEL, DIS, COUNT, CP, true>(cb, heads, a, PWb, base_b, row_scale_b, s, ln.n_glob, dd, K, Kmin, Kmax, cnt);
-  else
-    run_calls<MODEL, DIS, COUNT, CP, false>(cb, heads, a, PWb, base_b, row_scale_b, s, ln.n_glob, dd, K, Kmin, Kmax, cnt);
+  if (TABLE && heads) {
+    if (kLeft && a.left) calls(Flag<TABLE>{}, Flag<kLeft>{});
+    else calls(Flag<TABLE>{}, No{});
+  } else {
+    if (kLeft && a.left) calls(No{}, Flag<kLeft>{});
+    else calls(No{}, No{});
+  }
   attempts_fence();
+  cnt.a += hops.a - hops.b;
+  cnt.b += hops.b;
 }
 
 }  // namespace

@@ -44,6 +44,10 @@ struct Rates {
   int32_t pb, qb, pb_slow, qb_slow;
 };
 
+// Entries of a sample's table of heads: every call of the largest count, and
+// the one drawn ahead of it.
+constexpr uint32_t domain_calls(uint32_t ptab_klo, uint32_t ptab_n) { return (ptab_klo + ptab_n) / 4u + 3u; }
+
 inline int32_t hop_bound(uint32_t t) {
   return static_cast<int32_t>(0x80000000u + (t == 0xFFFFFFFFu ? (1u << 30) : (t >> 2)));
 }
@@ -114,7 +118,10 @@ struct DomainLaunch {
   uint32_t cluster;        // CTAs per sample: 1 = resident in one CTA, 2..16 = a thread-block cluster
   uint32_t Gc;             // cluster tier: columns per CTA (the last CTA may hold fewer)
   uint32_t lane_sort;      // resident tier: warps run domains of similar Poisson count (results unchanged)
-  uint32_t heads;          // resident tier with the lane sort: entries of a sample's table of heads (0 = no table)
+  uint32_t heads;          // entries of a sample's table of heads (0 = no table; see asep_domain.cuh)
+  uint32_t heads_at;       // cluster and streamed tiers: byte offset of the table in shared memory
+  uint32_t left;           // ring: left hops are possible
+  uint32_t inverse;        // all ones: plane 0 of the columns in shared memory holds the sites' complement
   uint32_t sca_kmax;       // SCA: random planes that decide every threshold (20 - fewest trailing zeros)
   Rates rates;
   uint64_t seed;
@@ -275,6 +282,7 @@ cudaError_t launch_advance_batch(const DomainLaunch* jobs, uint32_t n_jobs, cuda
 cudaError_t launch_set_clock(Clock* clock, uint64_t sweep, uint32_t next_time, cudaStream_t st);
 // Occupancy of the persistent kernel (CTAs per SM) for a block size and shared memory.
 int batch_ctas_per_sm(uint32_t threads, size_t smem);
+cudaError_t warm_advance_batch(cudaStream_t st);
 // Empty launches of the batch kernels (code loaded, local memory sized); `queue` is a device counter.
 cudaError_t warm_batch_kernels(uint32_t* queue, cudaStream_t st);
 cudaError_t launch_serial(const SerialLaunch& a, uint32_t model, uint32_t dis, cudaStream_t st);

@@ -126,6 +126,8 @@ __global__ void __launch_bounds__(1024) k_stream(const DomainLaunch a, uint32_t 
       if (part2) bulk_g2s(stage + p * SW + part1, base, part2 * 4u, &bar);
     }
   }
+  uint4* heads = reinterpret_cast<uint4*>(smem_raw + a.heads_at);  // while the copies are in flight
+  for (uint32_t i = threadIdx.x; i < a.heads; i += blockDim.x) heads[i] = domain_head(s, i, n_glob, a.ks);
   for (uint32_t i = threadIdx.x; i < a.ptab_n; i += blockDim.x) tab[i] = a.ptab[i];
   const bool done = mbar_wait_bounded(&bar, 0);
   if (__syncthreads_or(!done)) {  // copies did not complete: report, let them land, give up
@@ -141,7 +143,7 @@ __global__ void __launch_bounds__(1024) k_stream(const DomainLaunch a, uint32_t 
       const uint32_t* st = stage + p * SW + off;
       for (uint32_t r = 0; r <= R2; ++r) {
         const uint32_t f = c * R2 + r;
-        cols[p * PW + r * Cp + c] = sh ? __funnelshift_r(st[f], st[f + 1], sh) : st[f];
+        cols[p * PW + r * Cp + c] = (sh ? __funnelshift_r(st[f], st[f + 1], sh) : st[f]) ^ plane_inverse(a, p);
       }
     }
   }
@@ -157,7 +159,7 @@ __global__ void __launch_bounds__(1024) k_stream(const DomainLaunch a, uint32_t 
   ln.n_glob = n_glob;
   ln.active = c < Cn;
   Cnt cnt;
-  run_phase<MODEL, DIS, COUNT, 0, PHASE, false>(cols, nullptr, false, nullptr, false, a, tab, PW, s, ln, cnt);
+  run_phase<MODEL, DIS, COUNT, 0, PHASE, true>(cols, nullptr, false, a.heads ? heads : nullptr, false, a, tab, PW, s, ln, cnt);
   __syncthreads();
   if (PHASE == 1) {  // the last bond of column c reached row 0 of column c + 1 through its mirror row
     if (c + 1 < Cn) {
@@ -178,11 +180,12 @@ __global__ void __launch_bounds__(1024) k_stream(const DomainLaunch a, uint32_t 
     const uint32_t* st = stage + p * SW + off;
     uint32_t* dst_plane = a.state + (static_cast<size_t>(sample) * NOCC + p) * W;
     const uint32_t* cp = cols + p * PW;
+    const uint32_t inv = plane_inverse(a, p);
     for (uint32_t k = threadIdx.x; k < N; k += blockDim.x) {
       const uint32_t orig = st[k];
       uint32_t hi, lo;
       if (k <= last_f) {
-        const uint32_t fk = k < last_f ? cp[(k & (R2 - 1)) * Cp + (k >> a.logR2)] : cp[R2 * Cp + (Cn - 1)];
+        const uint32_t fk = (k < last_f ? cp[(k & (R2 - 1)) * Cp + (k >> a.logR2)] : cp[R2 * Cp + (Cn - 1)]) ^ inv;
         hi = fk << sh;
       } else {
         hi = orig & ~low;
@@ -191,7 +194,7 @@ __global__ void __launch_bounds__(1024) k_stream(const DomainLaunch a, uint32_t 
         lo = 0;
       } else if (k >= 1 && k - 1 <= last_f) {
         const uint32_t f = k - 1;
-        const uint32_t fk = f < last_f ? cp[(f & (R2 - 1)) * Cp + (f >> a.logR2)] : cp[R2 * Cp + (Cn - 1)];
+        const uint32_t fk = (f < last_f ? cp[(f & (R2 - 1)) * Cp + (f >> a.logR2)] : cp[R2 * Cp + (Cn - 1)]) ^ inv;
         lo = fk >> (32u - sh);
       } else {
         lo = orig & low;
