@@ -28,16 +28,15 @@
  *   ASEP_SCHED_SERIAL  plain random-sequential update (RSU, paper sec. 2.1):
  *                      per sweep L (two lanes: 2L) attempts on uniformly drawn
  *                      bonds; L a power of two.  Two plans, both giving the
- *                      sequential result: one CTA per sample, which runs a
- *                      sweep's attempts in rounds, each attempt once every
- *                      earlier attempt sharing a site with it has run (the
- *                      automatic plan when the lattice and a sweep's draws
- *                      fit 200 KB of shared memory -- a ring of up to 16384
- *                      sites, two lanes of up to 8192 -- and the samples
- *                      number at most four per SM); or one warp per sample, which
- *                      applies each batch of 32 consecutive attempts up to
- *                      the first one that shares a site with an earlier one
- *                      of the batch.
+ *                      sequential result: one CTA or one warp per sample.
+ *                      Both keep a window of the earliest attempts not yet
+ *                      done and go in rounds, each running every attempt of
+ *                      the window all of whose earlier site-sharing attempts
+ *                      are done.  One CTA (a window of 512) is the automatic
+ *                      plan when lattice and tables fit 200 KB of shared
+ *                      memory -- a ring of up to 16384 sites, two lanes of up
+ *                      to 8192 -- and the samples number at most six per SM
+ *                      (three per SM on rings of less than 4096 sites).
  *   ASEP_SCHED_DOMAIN  two-phase Poisson-domain RSU (no paper counterpart; the
  *                      paper's GPU schedule is a two-sub-lattice cellular
  *                      automaton).  Per sweep a random offset splits the ring

@@ -278,12 +278,14 @@ size_t sca_parts_bytes(const asep_ctx* ctx) {
 // force_cluster: 0 = choose, 1 = resident only, n > 1 = exactly n CTAs per
 // sample.  force_spc: samples per CTA for the resident plan (0 = choose).
 // The plan changes only the launch shape, never the results.
-// Serial-schedule plan.  kSerialRounds: one CTA per sample, the sweep's
-// attempts in dependency rounds (when the lattice and the sweep's draws fit
-// shared memory); kSerialWarp: one warp per sample.  force: 0 = the rounds
-// plan when it applies and the samples number at most four per SM (measured
-// on rings of 4096 sites: 4.6x the warp plan at 8 samples and at 152, 0.77x
-// at 1024, where the warps alone fill the GPU), else the warp plan.
+// Serial-schedule plan.  kSerialRounds: one CTA per sample (when lattice and
+// tables fit shared memory); kSerialWarp: one warp per sample.  force: 0 = the
+// CTA plan when it applies and the samples number at most six per SM, or three
+// per SM below 4096 sites, where its rounds are short of attempts; else the
+// warp plan, whose warps then fill the SMs.  Both, us per sweep: 152 rings of
+// 1024 / 4096 / 16384 sites 2.2, 4.9, 17 by CTAs and 7.6, 29, 118 by warps;
+// 456 of 1024 6.5 and 7.6, 608 8.7 and 7.6; 912 of 4096 29.2 and 33.5, 1216
+// 38.9 and 33.6; 912 of 16384 102 and 134, 1216 136 and 135.
 int plan_serial(asep_ctx* ctx, uint32_t force) {
   const uint32_t model = ctx->p.model, dis = ctx->p.dis_kind;
   const size_t smem = serial_rounds_smem_bytes(model, dis, ctx->L);
@@ -296,7 +298,7 @@ int plan_serial(asep_ctx* ctx, uint32_t force) {
     (void)cudaGetLastError();
     sms = 1;
   }
-  const bool few = ctx->S <= 4u * static_cast<uint32_t>(sms);
+  const bool few = ctx->S <= (ctx->L >= 4096 ? 6u : 3u) * static_cast<uint32_t>(sms);
   if (force == kSerialRounds || (force == 0 && smem > 0 && few)) {
     ctx->cluster = kSerialRounds;
     ctx->spc = 1;
@@ -935,7 +937,7 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
       a.state = ctx->d_state;
       a.mask = ctx->d_mask;
       a.rates = rates(ctx);
-      a.seed = ctx->p.seed;
+      a.ks = key_schedule(ctx->p.seed);
       a.n_sweeps = static_cast<uint32_t>(n);
       a.clock = ctx->d_clock;
       a.times = ctx->d_times;

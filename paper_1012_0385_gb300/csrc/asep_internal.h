@@ -142,7 +142,7 @@ struct SerialLaunch {
   uint32_t* state;
   const uint32_t* mask;
   Rates rates;
-  uint64_t seed;
+  KeySchedule ks;          // round keys of the seed
   uint32_t n_sweeps;
   Clock* clock;
   const uint64_t* times;
