@@ -215,14 +215,14 @@ __global__ void __launch_bounds__(1024) k_cluster(const DomainLaunch a) {
     nxt = t;
     R_cur = o;
     __syncthreads();
-    run_phase<MODEL, DIS, COUNT, 0, 0, true>(cur, nullptr, false, heads, false, a, tab, PW, s, ln, cnt);
+    run_phase<MODEL, DIS, COUNT, 0, 0, true>(cur, nullptr, false, heads, false, a, tab, PW, s, ln, cnt, a.G, a.C);
     cl.sync();
     if (ln.active) {
 #pragma unroll
       for (uint32_t p = 0; p < NP; ++p)
         cur[p * PW + R2 * Cp + ln.c] = *cl_word(cl, cur, p, PW, 0, Cp, gn, Gc, my_rank);
     }
-    run_phase<MODEL, DIS, COUNT, 0, 1, true>(cur, nullptr, false, heads, false, a, tab, PW, s, ln, cnt);
+    run_phase<MODEL, DIS, COUNT, 0, 1, true>(cur, nullptr, false, heads, false, a, tab, PW, s, ln, cnt, a.G, a.C);
     cl.sync();
     if (ln.active) {
 #pragma unroll

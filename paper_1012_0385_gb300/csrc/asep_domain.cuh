@@ -241,9 +241,11 @@ __device__ __forceinline__ void run_calls(uint32_t base, const uint4* heads, con
 // warp w runs the domains of rank w.  A domain's attempts are the same
 // whichever thread runs them, and a thread stays in its own sample and bank,
 // so results and bank mapping are unchanged; only the slots a warp wastes
-// shrink.  `scr` is the idle realign buffer (overwritten by the next realign).
-// The cluster tier passes sort = false: there other CTAs may still read that
-// buffer remotely during the first phase.
+// shrink.  G, C: the columns of the thread's sample and of the group (a
+// streamed tile: both its own).  `scr` is the idle realign buffer (overwritten
+// by the next realign) or the streamed tier's staged words.  The cluster tier
+// passes sort = false: there other CTAs may still read that buffer remotely
+// during the first phase.
 //
 // heads: the sample's table of heads, or nullptr.  fill: the table is formed
 // here (the first phase of a sweep), in the idle buffer behind the sort's
@@ -251,7 +253,7 @@ __device__ __forceinline__ void run_calls(uint32_t base, const uint4* heads, con
 template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP, uint32_t PHASE, bool TABLE>
 __device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sort, uint4* heads, bool fill,
                                           const DomainLaunch& a, const uint32_t* tab, uint32_t PW, uint64_t s,
-                                          const Lane& ln, Cnt& cnt) {
+                                          const Lane& ln, Cnt& cnt, uint32_t G, uint32_t C) {
   const uint32_t d = 2 * ln.g + PHASE;
   uint4 x0 = make_uint4(0u, 0u, 0u, 0u);
   uint32_t K = 0;
@@ -261,8 +263,8 @@ __device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sor
     x0 = ds.draw(0, a.ks);
     K = poisson_count(tab, a.ptab_n, a.ptab_klo, x0.x);
   }
-  if (fill && ln.c < a.C)
-    for (uint32_t c = ln.g; c < a.heads; c += a.G) heads[c] = domain_head(s, c, ln.n_glob, a.ks);
+  if (fill && ln.c < C)
+    for (uint32_t c = ln.g; c < a.heads; c += G) heads[c] = domain_head(s, c, ln.n_glob, a.ks);
   if (fill && !sort) __syncthreads();
   const uint32_t cp = CP ? CP : a.Cp;
   uint32_t col = ln.c;  // the column (domain pair) this thread runs
@@ -270,7 +272,7 @@ __device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sor
   if (sort) {
     // Only the group's own columns (c < C) take part: a persistent CTA may be
     // wider than the group, and its extra threads keep K = 0 and no column.
-    const bool in_group = ln.c < a.C;
+    const bool in_group = ln.c < C;
     uint32_t* sK = scr;
     uint32_t* sPerm = scr + cp;
     uint32_t* sX = scr + 2 * cp;
@@ -284,7 +286,7 @@ __device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sor
     if (in_group) {
       const uint32_t lane = ln.c & 31u;
       uint32_t rank = 0;
-      for (uint32_t q = ln.col0 + lane; q < ln.col0 + a.G; q += 32) {
+      for (uint32_t q = ln.col0 + lane; q < ln.col0 + G; q += 32) {
         const uint32_t kq = sK[q];
         rank += (kq < K || (kq == K && q < ln.c)) ? 1u : 0u;
       }

@@ -360,10 +360,12 @@ __device__ __forceinline__ void run_group(const DomainLaunch& a, uint32_t group,
     __syncthreads();
     uint4* heads =
         a.heads ? reinterpret_cast<uint4*>(nxt + (a.lane_sort ? 5u * Cp : 0u)) + s_loc * a.heads : nullptr;
-    run_phase<MODEL, DIS, COUNT, CP, 0, true>(cur, nxt, a.lane_sort != 0, heads, a.heads != 0, a, tab, PW, s, ln, cnt);
+    run_phase<MODEL, DIS, COUNT, CP, 0, true>(cur, nxt, a.lane_sort != 0, heads, a.heads != 0, a, tab, PW, s, ln, cnt,
+                                              a.G, a.C);
     __syncthreads();
     if (ln.active) mirror_in<NP>(cur, a, PW, ln);
-    run_phase<MODEL, DIS, COUNT, CP, 1, true>(cur, nxt, a.lane_sort != 0, heads, false, a, tab, PW, s, ln, cnt);
+    run_phase<MODEL, DIS, COUNT, CP, 1, true>(cur, nxt, a.lane_sort != 0, heads, false, a, tab, PW, s, ln, cnt, a.G,
+                                              a.C);
     __syncthreads();
     if (ln.active) mirror_out<NOCC>(cur, a, PW, ln);
     __syncthreads();

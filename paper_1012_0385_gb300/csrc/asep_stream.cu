@@ -159,7 +159,13 @@ __global__ void __launch_bounds__(1024) k_stream(const DomainLaunch a, uint32_t 
   ln.n_glob = n_glob;
   ln.active = c < Cn;
   Cnt cnt;
-  run_phase<MODEL, DIS, COUNT, 0, PHASE, true>(cols, nullptr, false, a.heads ? heads : nullptr, false, a, tab, PW, s, ln, cnt);
+  // The lane sort's scratch lies in the staged words: of those only the first and the last two of the tile are read
+  // again (k = 0 at stage[off], off <= 3, and the last two, from stage[off + R2 Cn] on).  Tiles too short for it run
+  // unsorted.  16 rings of 2^24, us per sweep by tile width, without and with the sort: 64 columns 416 and 417 (two
+  // domains a bank), 128 411 and 397, 256 421 and 406, 512 437 and 410.
+  uint32_t* scr = stage + 4;
+  run_phase<MODEL, DIS, COUNT, 0, PHASE, true>(cols, scr, 4 + 5 * Cp <= off + R2 * Cn, a.heads ? heads : nullptr, false, a,
+                                               tab, PW, s, ln, cnt, Cn, Cn);
   __syncthreads();
   if (PHASE == 1) {  // the last bond of column c reached row 0 of column c + 1 through its mirror row
     if (c + 1 < Cn) {
@@ -182,7 +188,7 @@ __global__ void __launch_bounds__(1024) k_stream(const DomainLaunch a, uint32_t 
     const uint32_t* cp = cols + p * PW;
     const uint32_t inv = plane_inverse(a, p);
     for (uint32_t k = threadIdx.x; k < N; k += blockDim.x) {
-      const uint32_t orig = st[k];
+      const uint32_t orig = st[k];  // meaningful at k = 0 and k >= N - 2
       uint32_t hi, lo;
       if (k <= last_f) {
         const uint32_t fk = (k < last_f ? cp[(k & (R2 - 1)) * Cp + (k >> a.logR2)] : cp[R2 * Cp + (Cn - 1)]) ^ inv;
