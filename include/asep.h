@@ -297,13 +297,16 @@ int asep_get_info(const asep_ctx* ctx, asep_info* info);
 
 /* Choose the launch plan of a context (the autotuner's knob; results never
  * depend on it).  Serial schedule: cluster 0 = automatic, 1 = one CTA per
- * sample running each sweep in dependency rounds (ASEP_ERR_INVALID beyond
- * 32768 attempts per sweep or 200 KB of shared memory), 2 = one warp per
- * sample; samples_per_group 0.  SCA: cluster 0 =
- * automatic, 1 = the ring in one CTA's shared memory (ASEP_ERR_INVALID when
- * it does not fit), 32 = streamed from global memory; samples_per_group 0.
- * Domain schedule: cluster 0 = automatic, 1 = whole samples in
- * one CTA, 2/4/8/16 = each sample spread over that many CTAs of a
+ * sample (ASEP_ERR_INVALID beyond 32768 attempts per sweep or 200 KB of
+ * shared memory), 2 = one warp per sample; samples_per_group 0.  SCA: cluster
+ * 0 = automatic, 1 or 32 = the names of short and long rings (1 gives
+ * ASEP_ERR_INVALID for a ring beyond one CTA's shared memory); both run by
+ * the same tiles, a warp each; samples_per_group 0.
+ * Domain schedule: cluster 0 = automatic (whole samples in one CTA where they
+ * fit; launches of few samples of at least 256 columns are then spread over
+ * clusters of 2 to 16 CTAs, and batches run such launches side by side; beyond
+ * one CTA the smallest cluster that holds a sample, or up to 16 CTAs where few
+ * samples leave SMs idle), 1 = whole samples in one CTA, 2/4/8/16 = each sample spread over that many CTAs of a
  * thread-block cluster (columns of 2D sites split evenly), 32 = streamed: the
  * lattice stays in global memory and tiles of columns pass through shared
  * memory once per phase (the automatic choice when a sample fits neither one

@@ -61,6 +61,11 @@ struct asep_ctx {
   uint32_t cluster = 1, Gc = 0;  // cluster tier: CTAs per sample, columns per CTA (kStreamTier: streamed)
   uint32_t tiles = 0;             // streamed tier: tiles per sample
   uint32_t heads_at = 0;          // cluster and streamed tiers: offset of the table of heads in shared memory (0 = none)
+  // the cluster plan an automatic resident plan's launches take where the samples are few (cluster = 0: none)
+  struct ClusterPlan {
+    uint32_t cluster = 0, Gc = 0, Cp = 0, heads_at = 0;
+    size_t smem = 0;
+  } spread;
   uint32_t* d_err = nullptr;      // device flag: a streamed tile's copy wait gave up
   uint32_t fault = ASEP_FAULT_NONE;  // injected fault (asep_inject_fault)
   size_t smem = 0;
@@ -279,6 +284,16 @@ size_t sca_parts_bytes(const asep_ctx* ctx) {
 // force_cluster: 0 = choose, 1 = resident only, n > 1 = exactly n CTAs per
 // sample.  force_spc: samples per CTA for the resident plan (0 = choose).
 // The plan changes only the launch shape, never the results.
+int sm_count() {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) {
+    (void)cudaGetLastError();
+    sms = 1;
+  }
+  return sms;
+}
+
 // Serial-schedule plan.  kSerialRounds: one CTA per sample (when lattice and
 // tables fit shared memory); kSerialWarp: one warp per sample.  force: 0 = the
 // CTA plan when it applies and the samples number at most six per SM, or three
@@ -293,12 +308,7 @@ int plan_serial(asep_ctx* ctx, uint32_t force) {
   if (force == kSerialRounds && smem == 0)
     return fail(ctx, ASEP_ERR_INVALID, "the one-CTA serial plan needs at most %u attempts per sweep and 200 KB of "
                 "shared memory", kSerialRoundsMaxAttempts);
-  int dev = 0, sms = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                               cudaSuccess || sms <= 0) {
-    (void)cudaGetLastError();
-    sms = 1;
-  }
+  const int sms = sm_count();
   const bool few = ctx->S <= (ctx->L >= 4096 ? 6u : 3u) * static_cast<uint32_t>(sms);
   if (force == kSerialRounds || (force == 0 && smem > 0 && few)) {
     ctx->cluster = kSerialRounds;
@@ -315,6 +325,50 @@ int plan_serial(asep_ctx* ctx, uint32_t force) {
     ctx->blocks = (ctx->S + warps - 1) / warps;
   }
   return ASEP_OK;
+}
+
+// The cluster plan with nc CTAs per sample, if it fits the device.
+bool cluster_plan(const asep_ctx* ctx, uint32_t nc, asep_ctx::ClusterPlan* out) {
+  const uint32_t dis = ctx->p.dis_kind, ptab_n = static_cast<uint32_t>(ctx->ptab.size());
+  const uint32_t Gc = (ctx->G + nc - 1) / nc;
+  if (Gc > 1024 || (ctx->G + Gc - 1) / Gc != nc) return false;  // every CTA of the cluster holds columns
+  const uint32_t Cp = (Gc + 31) / 32 * 32;
+  const size_t smem = domain_smem_bytes(ctx->p.model, dis, ctx->R2, Cp, ptab_n, Cp);
+  if (smem + 64 > 227 * 1024 || Cp > 1024 || cluster_fits(ctx->p.model, dis, nc, Cp, smem) <= 0) return false;
+  // the table of random heads behind the rest, where that still fits
+  const size_t at = (smem + 15) & ~static_cast<size_t>(15);
+  const size_t with = at + 16ull * domain_calls(ctx->ptab_klo, ptab_n);
+  const bool table = with + 64 <= 227 * 1024 && cluster_fits(ctx->p.model, dis, nc, Cp, with) > 0;
+  out->cluster = nc;
+  out->Gc = Gc;
+  out->Cp = Cp;
+  out->heads_at = table ? static_cast<uint32_t>(at) : 0u;
+  out->smem = table ? with : smem;
+  return true;
+}
+
+// Few samples leave most SMs idle: twice the CTAs per sample then, while each
+// keeps 128 columns and the clusters find room side by side -- 7/8 of the SMs
+// for clusters of 2 and 4, 5/9 for 8 and 16, of which a GPC holds one or two.
+// us per sweep by CTAs per sample: one ring of 2^18 1: 54, 2: 42, 4: 35, 8: 35;
+// one of 2^19 1: 98, 2: 60, 4: 42, 8: 36; 8 of 2^20 2: 109, 4: 61, 8: 43, 16: 42;
+// 32 of 655360 2: 72, 4: 50, 8: 52; 64 of them 2: 72, 4: 80; 16 of 2^21 4: 110,
+// 8: 113; 4 of 2^22 8: 110, 16: 62; 5 pairs of lanes of 1626112 8: 121, 16: 80.
+bool spreads(const asep_ctx* ctx, uint32_t nc, uint32_t sms) {
+  const uint64_t ctas = static_cast<uint64_t>(ctx->S) * nc;
+  return nc <= 16 && ctx->G >= 128ull * nc && (nc <= 4 ? 8 * ctas <= 7ull * sms : 9 * ctas <= 5ull * sms);
+}
+
+// The cluster plan for the launches of a resident plan chosen automatically
+// (info and batches' limits stay those of the resident plan).
+void plan_spread(asep_ctx* ctx, bool automatic) {
+  ctx->spread = asep_ctx::ClusterPlan{};
+  if (!automatic || ctx->p.schedule != ASEP_SCHED_DOMAIN || ctx->cluster != 1 || ctx->spc != 1) return;
+  const uint32_t sms = static_cast<uint32_t>(sm_count());
+  for (uint32_t nc = 2; spreads(ctx, nc, sms); nc *= 2) {
+    asep_ctx::ClusterPlan next;
+    if (cluster_plan(ctx, nc, &next)) ctx->spread = next;
+  }
 }
 
 // Automatic tile width of the streamed tier, in columns (one thread each).
@@ -356,26 +410,22 @@ int plan_domain(asep_ctx* ctx, uint32_t force_cluster, uint32_t force_spc) {
     if (!placed && (force_cluster == 1 || force_spc))
       return fail(ctx, ASEP_ERR_INVALID, "the requested resident plan does not fit one CTA");
   }
-  for (uint32_t nc = force_cluster > 1 ? force_cluster : 2; !placed && nc <= 16 && force_cluster != kStreamTier;
-       nc *= 2) {
-    const uint32_t Gc = static_cast<uint32_t>((G + nc - 1) / nc);
-    const bool ok = Gc <= 1024 && (G + Gc - 1) / Gc == nc;  // every CTA of the cluster holds columns
-    const uint32_t Cp = (Gc + 31) / 32 * 32;
-    const size_t smem = domain_smem_bytes(ctx->p.model, dis, ctx->R2, Cp, ptab_n, Cp);
-    if (ok && smem + 64 <= 227 * 1024 && Cp <= 1024 && cluster_fits(ctx->p.model, dis, nc, Cp, smem) > 0) {
-      // the table of random heads behind the rest, where that still fits
-      const size_t at = (smem + 15) & ~static_cast<size_t>(15), with = at + 16ull * calls;
-      const bool table = with + 64 <= 227 * 1024 && cluster_fits(ctx->p.model, dis, nc, Cp, with) > 0;
-      ctx->heads_at = table ? static_cast<uint32_t>(at) : 0u;
+  uint32_t sms = 0;
+  for (uint32_t nc = force_cluster > 1 ? force_cluster : 2; nc <= 16 && force_cluster != kStreamTier; nc *= 2) {
+    if (placed && (ctx->cluster == 1 || !spreads(ctx, nc, sms))) break;
+    asep_ctx::ClusterPlan plan;
+    if (cluster_plan(ctx, nc, &plan)) {
+      ctx->heads_at = plan.heads_at;
       ctx->cluster = nc;
       ctx->spc = 1;
-      ctx->C = Gc;
-      ctx->Gc = Gc;
-      ctx->Cp = Cp;
-      ctx->threads = Cp;
-      ctx->smem = table ? with : smem;
+      ctx->C = plan.Gc;
+      ctx->Gc = plan.Gc;
+      ctx->Cp = plan.Cp;
+      ctx->threads = plan.Cp;
+      ctx->smem = plan.smem;
       ctx->blocks = ctx->S;
       placed = true;
+      sms = static_cast<uint32_t>(sm_count());
     }
     if (force_cluster > 1) break;
   }
@@ -520,7 +570,8 @@ int record_now(asep_ctx* ctx, uint32_t slot) {
   return ASEP_OK;
 }
 
-DomainLaunch domain_desc(const asep_ctx* ctx, uint32_t n) {
+// A launch of n sweeps; spread: by the cluster plan ctx->spread.
+DomainLaunch domain_desc(const asep_ctx* ctx, uint32_t n, bool spread = false) {
   DomainLaunch a{};
   a.geo = geometry(ctx);
   a.model = ctx->p.model;
@@ -538,20 +589,20 @@ DomainLaunch domain_desc(const asep_ctx* ctx, uint32_t n) {
   a.row_bits = (ctx->D - 1) & ~31u;
   a.G = ctx->G;
   a.spc = ctx->spc;
-  a.C = ctx->C;
-  a.Cp = ctx->Cp;
+  a.C = spread ? ctx->spread.Gc : ctx->C;
+  a.Cp = spread ? ctx->spread.Cp : ctx->Cp;
   a.n_groups = ctx->blocks;
-  a.cluster = ctx->cluster;
-  a.Gc = ctx->Gc;
+  a.cluster = spread ? ctx->spread.cluster : ctx->cluster;
+  a.Gc = spread ? ctx->spread.Gc : ctx->Gc;
+  a.heads_at = spread ? ctx->spread.heads_at : ctx->heads_at;
   {
     // every warp inside one sample, and the idle realign buffer holds 5 words per column
     const uint32_t np = (ctx->p.model == ASEP_MODEL_TWO_LANE ? 2u : 1u) + dis_planes(ctx->p.dis_kind);
-    a.lane_sort = (ctx->cluster <= 1 && ctx->G % 32 == 0 && np * (ctx->R2 + 1) >= 5) ? 1u : 0u;
+    a.lane_sort = (a.cluster <= 1 && ctx->G % 32 == 0 && np * (ctx->R2 + 1) >= 5) ? 1u : 0u;
     // ... and, behind them, a table of four words per call for each of its samples (from some 25 columns on)
     const uint32_t calls = domain_calls(a.ptab_klo, a.ptab_n);
     const bool fits = 4ull * calls * ctx->spc <= (np * (ctx->R2 + 1ull) - (a.lane_sort ? 5u : 0u)) * ctx->Cp;
-    a.heads = ctx->cluster <= 1 ? (fits ? calls : 0u) : (ctx->heads_at ? calls : 0u);
-    a.heads_at = ctx->heads_at;
+    a.heads = a.cluster <= 1 ? (fits ? calls : 0u) : (a.heads_at ? calls : 0u);
   }
   a.rates = rates(ctx);
   a.left = ctx->p.model == ASEP_MODEL_RING && (a.rates.q || a.rates.q_slow) ? 1u : 0u;
@@ -796,6 +847,7 @@ int asep_create(const asep_params* params, asep_ctx** out) {
   };
   rc = plan_context(ctx, params);
   if (rc != ASEP_OK) return bail(rc);
+  plan_spread(ctx, true);
 
   // device memory (planned_device_bytes lists the same sizes)
   const size_t state_words = static_cast<size_t>(ctx->S) * ctx->planes * ctx->W;
@@ -929,6 +981,8 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
       b.stall = ctx->fault == ASEP_FAULT_BALANCE_STALL ? 1u : 0u;
       e = launch_domain_balanced(domain_desc(ctx, static_cast<uint32_t>(n)), b, ctx->threads, ctx->smem,
                                  ctx->stream);
+    } else if (ctx->p.schedule == ASEP_SCHED_DOMAIN && ctx->spread.cluster) {
+      e = launch_cluster(domain_desc(ctx, static_cast<uint32_t>(n), true), ctx->spread.Cp, ctx->spread.smem, ctx->stream);
     } else if (ctx->p.schedule == ASEP_SCHED_DOMAIN) {
       e = launch_domain(domain_desc(ctx, static_cast<uint32_t>(n)), ctx->threads, ctx->smem, ctx->stream);
     } else {
@@ -1121,7 +1175,7 @@ int asep_disorder(asep_ctx* ctx, uint32_t* words, size_t n_words) {
 }  // extern "C"
 
 // Streams for the cluster-tier contexts of a step.
-constexpr uint32_t kAuxStreams = 8;
+constexpr uint32_t kAuxStreams = 16;
 
 struct asep_batch {
   cudaStream_t stream = nullptr;
@@ -1160,15 +1214,21 @@ int bfail(asep_batch* b, int code, const char* fmt, ...) {
 // upload them, and compute the launch shape.  n[i] <= the context's cap.
 int batch_prepare(asep_batch* b, asep_ctx* const* ctxs, const uint32_t* n, uint32_t nj, uint32_t* n_items_out,
                   uint32_t* threads_out, uint32_t* ctas_out, size_t* smem_out) {
-  uint32_t threads = 32;
-  for (uint32_t j = 0; j < nj; ++j)
-    if (ctxs[j]->cluster == 1) threads = std::max(threads, ctxs[j]->threads);
+  uint32_t threads = 32, own = 32;  // of the resident plans; of those whose launches are not spread
+  for (uint32_t j = 0; j < nj; ++j) {
+    if (ctxs[j]->cluster != 1) continue;
+    threads = std::max(threads, ctxs[j]->threads);
+    if (!ctxs[j]->spread.cluster) own = std::max(own, ctxs[j]->threads);
+  }
   if (b->threads_req) {
     if (b->threads_req < threads || (b->threads_req & 31) || b->threads_req > 1024)
       return bfail(b, ASEP_ERR_INVALID, "threads %u: must be a multiple of 32 in [%u, 1024]", b->threads_req, threads);
-    threads = b->threads_req;
+    own = b->threads_req;
   }
+  const uint32_t widest = b->threads_req ? b->threads_req : threads;
+  threads = own;
   size_t smem = 0;
+  size_t n_groups = 0, most = 0;  // of the resident plans: what max_items and the 227 KB bound
   struct It {
     uint64_t cost;
     uint32_t code;
@@ -1178,27 +1238,29 @@ int batch_prepare(asep_batch* b, asep_ctx* const* ctxs, const uint32_t* n, uint3
   if (e != cudaSuccess) return bfail(b, ASEP_ERR_CUDA, "staging event: %s", cudaGetErrorString(e));
   for (uint32_t j = 0; j < nj; ++j) {
     const asep_ctx* c = ctxs[j];
-    b->h_jobs[j] = domain_desc(c, n[j]);
+    b->h_jobs[j] = domain_desc(c, n[j], c->spread.cluster != 0);
     if (c->cluster > 1) continue;  // cluster-tier contexts get their own cluster launch
+    if (n[j]) n_groups += c->blocks;
+    most = std::max(most, domain_smem_bytes(c->p.model, c->p.dis_kind, c->R2, c->Cp,
+                                            static_cast<uint32_t>(c->ptab.size()), widest));
+    if (c->spread.cluster) continue;  // and so do resident ones of few samples
     smem = std::max(smem, domain_smem_bytes(c->p.model, c->p.dis_kind, c->R2, c->Cp,
                                             static_cast<uint32_t>(c->ptab.size()), threads));
     if (n[j] == 0) continue;
     const uint64_t cost = static_cast<uint64_t>(n[j]) * c->spc * c->L * c->planes;
     for (uint32_t g = 0; g < c->blocks; ++g) items.push_back({cost, (j << kItemGroupBits) | g});
   }
-  if (items.size() > b->max_items)
-    return bfail(b, ASEP_ERR_INVALID, "%zu queue items exceed the batch's max_items %u", items.size(), b->max_items);
+  if (n_groups > b->max_items)
+    return bfail(b, ASEP_ERR_INVALID, "%zu queue items exceed the batch's max_items %u", n_groups, b->max_items);
   std::stable_sort(items.begin(), items.end(), [](const It& x, const It& y) { return x.cost > y.cost; });
   for (size_t i = 0; i < items.size(); ++i) b->h_items[i] = items[i].code;
   // the batch kernel's own static shared memory (item index, descriptor) shares the 227 KB opt-in
-  if (smem + sizeof(DomainLaunch) + 64 > 227 * 1024)
-    return bfail(b, ASEP_ERR_INVALID, "batch needs %zu bytes of shared memory", smem);
+  if (most + sizeof(DomainLaunch) + 64 > 227 * 1024)
+    return bfail(b, ASEP_ERR_INVALID, "batch needs %zu bytes of shared memory", most);
   int per_sm = batch_ctas_per_sm(threads, smem);
   if (per_sm <= 0) return bfail(b, ASEP_ERR_INVALID, "batch kernel does not fit (%u threads, %zu B)", threads, smem);
   if (b->ctas_per_sm_req) per_sm = std::min<int>(per_sm, static_cast<int>(b->ctas_per_sm_req));
-  int dev = 0, sms = 0;
-  cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  const int sms = sm_count();
   const uint32_t ctas = static_cast<uint32_t>(std::max<size_t>(1, std::min<size_t>(items.size(),
                                                                   static_cast<size_t>(per_sm) * sms)));
   if ((e = cudaMemcpyAsync(b->d_jobs, b->h_jobs, nj * sizeof(DomainLaunch), cudaMemcpyHostToDevice, b->stream)) !=
@@ -1267,18 +1329,18 @@ int order_out(asep_batch* b, asep_ctx* const* ctxs, uint32_t n) {
 int batch_step_enqueue(asep_batch* b, asep_ctx* const* ctxs, uint32_t nj, uint32_t n_items, uint32_t threads,
                        uint32_t ctas, size_t smem, cudaStream_t st) {
   cudaError_t e;
-  // Contexts of the cluster tier run as their own cluster launches on
-  // auxiliary streams forked from `st`, beside the persistent kernel and one
-  // another (their memory is their own), and are joined back before the clocks
-  // advance.  One launch is seldom more than a few clusters, each as long as
-  // its sweeps: on one stream they ran one after the other, 21.3 ms for the
-  // eight of a mix whose longest takes 4.5 ms and whose persistent kernel 7.4;
-  // on eight 7.4 ms for the whole step.  Longest first, each to the stream with
-  // the least to do.
+  // Contexts of the cluster tier, and spread ones, run as their own cluster
+  // launches on auxiliary streams forked from `st`, beside the persistent
+  // kernel and one another (their memory is their own), and are joined back
+  // before the clocks advance.  One launch is seldom more than a few clusters,
+  // each as long as its sweeps: on one stream the eight of a mix of 24 contexts
+  // ran one after the other, 21.3 ms; side by side 7.4 (the persistent kernel's
+  // two rings of 2^19), with those spread too 4.8.  Longest first, each to the
+  // stream with the least to do.
   std::vector<std::pair<uint64_t, uint32_t>> clusters;  // {rows of attempts a CTA goes through, context}
   for (uint32_t j = 0; j < nj; ++j)
-    if (ctxs[j]->cluster != 1 && b->h_jobs[j].n_sweeps)
-      clusters.emplace_back(static_cast<uint64_t>(b->h_jobs[j].n_sweeps) * (512u + ctxs[j]->threads), j);
+    if (b->h_jobs[j].cluster > 1 && b->h_jobs[j].n_sweeps)
+      clusters.emplace_back(static_cast<uint64_t>(b->h_jobs[j].n_sweeps) * (512u + b->h_jobs[j].Cp), j);
   std::stable_sort(clusters.begin(), clusters.end(), [](const auto& x, const auto& y) { return x.first > y.first; });
   const uint32_t used = static_cast<uint32_t>(std::min<size_t>(clusters.size(), kAuxStreams));
   uint64_t busy[kAuxStreams] = {};
@@ -1287,15 +1349,25 @@ int batch_step_enqueue(asep_batch* b, asep_ctx* const* ctxs, uint32_t nj, uint32
   for (uint32_t k = 0; k < used; ++k)
     if ((e = cudaStreamWaitEvent(b->aux_stream[k], b->fork, 0)) != cudaSuccess)
       return bfail(b, ASEP_ERR_CUDA, "fork: %s", cudaGetErrorString(e));
+  const auto persistent = [&] {
+    if (n_items && (e = launch_batch(b->d_jobs, b->d_items, n_items, b->d_queue, threads, ctas, smem, st)) !=
+                       cudaSuccess)
+      return bfail(b, ASEP_ERR_CUDA, "batch kernel: %s", cudaGetErrorString(e));
+    return static_cast<int>(ASEP_OK);
+  };
+  // A persistent kernel of few CTAs goes ahead of the clusters, which leave it no room for as long as they run
+  // (measured: 17 CTAs, the step 6.2 ms behind them and 4.8 ahead); one that could fill the SMs goes behind.
+  const bool first = 2 * ctas <= static_cast<uint32_t>(sm_count());
+  int rc = ASEP_OK;
+  if (first && (rc = persistent()) != ASEP_OK) return rc;
   for (const auto& [cost, j] : clusters) {
     const uint32_t k = static_cast<uint32_t>(std::min_element(busy, busy + used) - busy);
     busy[k] += cost;
-    if ((e = launch_cluster(b->h_jobs[j], ctxs[j]->threads, ctxs[j]->smem, b->aux_stream[k])) != cudaSuccess)
+    const size_t smem_j = ctxs[j]->cluster > 1 ? ctxs[j]->smem : ctxs[j]->spread.smem;
+    if ((e = launch_cluster(b->h_jobs[j], b->h_jobs[j].Cp, smem_j, b->aux_stream[k])) != cudaSuccess)
       return bfail(b, ASEP_ERR_CUDA, "cluster kernel of context %u: %s", j, cudaGetErrorString(e));
   }
-  if (n_items && (e = launch_batch(b->d_jobs, b->d_items, n_items, b->d_queue, threads, ctas, smem, st)) !=
-                     cudaSuccess)
-    return bfail(b, ASEP_ERR_CUDA, "batch kernel: %s", cudaGetErrorString(e));
+  if (!first && (rc = persistent()) != ASEP_OK) return rc;
   for (uint32_t k = 0; k < used; ++k)
     if ((e = cudaEventRecord(b->join[k], b->aux_stream[k])) != cudaSuccess ||
         (e = cudaStreamWaitEvent(st, b->join[k], 0)) != cudaSuccess)
@@ -1531,6 +1603,8 @@ int asep_set_plan(asep_ctx* ctx, uint32_t cluster, uint32_t samples_per_group) {
     ctx->heads_at = saved.heads_at;
     ctx->max_sweeps_per_launch = saved.max_sweeps_per_launch;
     ctx->err = msg;
+  } else {
+    plan_spread(ctx, cluster == 0 && samples_per_group == 0);
   }
   return rc;
 }
