@@ -15,25 +15,26 @@ namespace asep {
 namespace {
 
 // Runtime dispatch of one group to the matching instantiation.
+template <bool PIN>
 __device__ __forceinline__ void run_group_any(const DomainLaunch& a, uint32_t group, unsigned char* smem) {
   const uint64_t s0 = a.clock->sweep;
   const uint32_t cur = a.clock->next_time, n = a.n_sweeps;
   if (a.model == kTwoLane) {
-    if (a.dis == kDisTurning) run_group<kTwoLane, kDisTurning, true, 0>(a, group, smem, s0, cur, n);
-    else if (a.dis == kDisCrossing) run_group<kTwoLane, kDisCrossing, true, 0>(a, group, smem, s0, cur, n);
-    else run_group<kTwoLane, kDisNone, true, 0>(a, group, smem, s0, cur, n);
+    if (a.dis == kDisTurning) run_group<kTwoLane, kDisTurning, true, 0, PIN>(a, group, smem, s0, cur, n);
+    else if (a.dis == kDisCrossing) run_group<kTwoLane, kDisCrossing, true, 0, PIN>(a, group, smem, s0, cur, n);
+    else run_group<kTwoLane, kDisNone, true, 0, PIN>(a, group, smem, s0, cur, n);
   } else if (a.dis == kDisBimodal) {
-    if (a.count_hops) run_group<kRing, kDisBimodal, true, 0>(a, group, smem, s0, cur, n);
-    else run_group<kRing, kDisBimodal, false, 0>(a, group, smem, s0, cur, n);
+    if (a.count_hops) run_group<kRing, kDisBimodal, true, 0, PIN>(a, group, smem, s0, cur, n);
+    else run_group<kRing, kDisBimodal, false, 0, PIN>(a, group, smem, s0, cur, n);
   } else if (a.dis == kDisBimodalPQ) {
-    if (a.count_hops) run_group<kRing, kDisBimodalPQ, true, 0>(a, group, smem, s0, cur, n);
-    else run_group<kRing, kDisBimodalPQ, false, 0>(a, group, smem, s0, cur, n);
+    if (a.count_hops) run_group<kRing, kDisBimodalPQ, true, 0, PIN>(a, group, smem, s0, cur, n);
+    else run_group<kRing, kDisBimodalPQ, false, 0, PIN>(a, group, smem, s0, cur, n);
   } else if (a.Cp == 256) {
-    if (a.count_hops) run_group<kRing, kDisNone, true, 256>(a, group, smem, s0, cur, n);
-    else run_group<kRing, kDisNone, false, 256>(a, group, smem, s0, cur, n);
+    if (a.count_hops) run_group<kRing, kDisNone, true, 256, PIN>(a, group, smem, s0, cur, n);
+    else run_group<kRing, kDisNone, false, 256, PIN>(a, group, smem, s0, cur, n);
   } else {
-    if (a.count_hops) run_group<kRing, kDisNone, true, 0>(a, group, smem, s0, cur, n);
-    else run_group<kRing, kDisNone, false, 0>(a, group, smem, s0, cur, n);
+    if (a.count_hops) run_group<kRing, kDisNone, true, 0, PIN>(a, group, smem, s0, cur, n);
+    else run_group<kRing, kDisNone, false, 0, PIN>(a, group, smem, s0, cur, n);
   }
 }
 
@@ -55,7 +56,7 @@ __global__ void __maxnreg__(MAXT == 512 ? 104 : 64) k_batch(const DomainLaunch* 
     const uint32_t it = items[i];
     if (threadIdx.x == 0) desc = jobs[it >> kItemGroupBits];
     __syncthreads();
-    run_group_any(desc, it & (kItemMaxGroups - 1u), smem_raw);
+    run_group_any<MAXT == 512>(desc, it & (kItemMaxGroups - 1u), smem_raw);
   }
 }
 

@@ -231,6 +231,40 @@ __device__ __forceinline__ void run_calls(uint32_t base, const uint4* heads, con
   }
 }
 
+// A phase's view of its descriptor.  As a kernel parameter it lies in the
+// constant bank, whose words an instruction reads as operands.  A batch's CTA
+// holds it in shared memory, from where every Philox call loaded its 14 round
+// keys and the rates again; pinned, these are values of registers that the
+// compiler cannot load anew.  us per sweep of a batch of one context, of eight
+// rings of 4096, without and with: q = 0 38.5 -> 28.4, bimodal 48.7 -> 31.6, 39
+// pairs of lanes of 3840 with turning sites 54.6 -> 45.2.  Only in the class of
+// up to 512 threads: at 64 registers a thread they do not fit.
+template <bool PIN>
+struct HotFields {
+  const DomainLaunch& a;
+  __device__ __forceinline__ explicit HotFields(const DomainLaunch& d) : a(d) {}
+};
+__device__ __forceinline__ void pin(uint32_t& v) { asm volatile("" : "+r"(v)); }
+__device__ __forceinline__ void pin(int32_t& v) { asm volatile("" : "+r"(v)); }
+template <>
+struct HotFields<true> {
+  DomainLaunch a;
+  __device__ __forceinline__ explicit HotFields(const DomainLaunch& d) : a(d) {
+#pragma unroll
+    for (int r = 2; r < 10; ++r) {
+      pin(a.ks.x[r]);
+      pin(a.ks.y[r]);
+    }
+    pin(a.rates.pb);
+    pin(a.rates.qb);
+    pin(a.rates.pb_slow);
+    pin(a.rates.qb_slow);
+    pin(a.row_bits);
+    pin(a.logD);
+    pin(a.Cp);
+  }
+};
+
 // One half-domain phase of one sweep.  All threads of the block must call.
 //
 // Lane sort: the lanes of a warp run to the largest Poisson count of the
@@ -250,10 +284,12 @@ __device__ __forceinline__ void run_calls(uint32_t base, const uint4* heads, con
 // heads: the sample's table of heads, or nullptr.  fill: the table is formed
 // here (the first phase of a sweep), in the idle buffer behind the sort's
 // scratch, by the sample's threads.
-template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP, uint32_t PHASE, bool TABLE>
+template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP, uint32_t PHASE, bool TABLE, bool PIN = false>
 __device__ __forceinline__ void run_phase(uint32_t* cur, uint32_t* scr, bool sort, uint4* heads, bool fill,
-                                          const DomainLaunch& a, const uint32_t* tab, uint32_t PW, uint64_t s,
+                                          const DomainLaunch& desc, const uint32_t* tab, uint32_t PW, uint64_t s,
                                           const Lane& ln, Cnt& cnt, uint32_t G, uint32_t C) {
+  HotFields<PIN> hot(desc);
+  const DomainLaunch& a = hot.a;
   const uint32_t d = 2 * ln.g + PHASE;
   uint4 x0 = make_uint4(0u, 0u, 0u, 0u);
   uint32_t K = 0;

@@ -299,7 +299,7 @@ __device__ void record_extras(const uint32_t* cur, const DomainLaunch& a, uint32
 // reference lattice) may have been written by another CTA of the same launch
 // (the balanced kernel hands groups between CTAs): read them from L2
 // (ld.global.cg), never from a possibly stale L1 line.
-template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP>
+template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP, bool PIN = false>
 __device__ __forceinline__ void run_group(const DomainLaunch& a, uint32_t group, unsigned char* smem_raw,
                                           uint64_t s0, uint32_t cursor, uint32_t n_sweeps) {
   constexpr uint32_t NOCC = MODEL == kTwoLane ? 2u : 1u;
@@ -360,12 +360,12 @@ __device__ __forceinline__ void run_group(const DomainLaunch& a, uint32_t group,
     __syncthreads();
     uint4* heads =
         a.heads ? reinterpret_cast<uint4*>(nxt + (a.lane_sort ? 5u * Cp : 0u)) + s_loc * a.heads : nullptr;
-    run_phase<MODEL, DIS, COUNT, CP, 0, true>(cur, nxt, a.lane_sort != 0, heads, a.heads != 0, a, tab, PW, s, ln, cnt,
-                                              a.G, a.C);
+    run_phase<MODEL, DIS, COUNT, CP, 0, true, PIN>(cur, nxt, a.lane_sort != 0, heads, a.heads != 0, a, tab, PW, s, ln,
+                                                   cnt, a.G, a.C);
     __syncthreads();
     if (ln.active) mirror_in<NP>(cur, a, PW, ln);
-    run_phase<MODEL, DIS, COUNT, CP, 1, true>(cur, nxt, a.lane_sort != 0, heads, false, a, tab, PW, s, ln, cnt, a.G,
-                                              a.C);
+    run_phase<MODEL, DIS, COUNT, CP, 1, true, PIN>(cur, nxt, a.lane_sort != 0, heads, false, a, tab, PW, s, ln, cnt,
+                                                   a.G, a.C);
     __syncthreads();
     if (ln.active) mirror_out<NOCC>(cur, a, PW, ln);
     __syncthreads();
