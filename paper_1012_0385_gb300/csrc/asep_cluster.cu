@@ -151,8 +151,12 @@ __device__ void record_extras_cl(const cg::cluster_group& cl, const uint32_t* cu
   }
 }
 
+// One CTA per SM in the register budget: left to itself the compiler took 32
+// registers for plain rings, for a second CTA of 1024 threads that shared
+// memory never admits, and spilled 17.  us per sweep, before and after: one ring
+// of 2^18 31.9 -> 29.6, four of 2^22 62.8 -> 61.8.
 template <uint32_t MODEL, uint32_t DIS, bool COUNT>
-__global__ void __launch_bounds__(1024) k_cluster(const DomainLaunch a) {
+__global__ void __launch_bounds__(1024, 1) k_cluster(const DomainLaunch a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ long long cta_sums[4];
   constexpr uint32_t NOCC = MODEL == kTwoLane ? 2u : 1u;

@@ -84,9 +84,12 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 // One phase of one tile.  Grid: tiles x S CTAs, blockIdx.x = sample * tiles + tile.
 // stall: bytes the tile's copies announce beyond what they carry (0; a test
 // of the timeout path sets it, so that the wait for them runs out).
+// Registers: 32 or 35 for plain rings (at 64 the eight CTAs of 128 that stay on
+// an SM are 2 % slower than eleven), up to 64 where quenched planes would spill
+// at 32: 8 rings of 2^24 with both classes 761 -> 742 us per sweep.
 template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t PHASE>
-__global__ void __launch_bounds__(1024) k_stream(const DomainLaunch a, uint32_t tiles, uint32_t* err,
-                                                 uint32_t stall) {
+__global__ void __launch_bounds__(1024, MODEL == kRing && DIS == kDisNone ? 0 : 1)
+    k_stream(const DomainLaunch a, uint32_t tiles, uint32_t* err, uint32_t stall) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t bar;
   constexpr uint32_t NOCC = MODEL == kTwoLane ? 2u : 1u;
