@@ -122,8 +122,8 @@ class ClockSampler:
 KERNEL_SOURCES = {
     "domain": ("asep_kernels.cu", "asep_resident.cuh", "asep_domain.cuh", "asep_device.cuh", "asep_internal.h"),
     "domain_bal": ("asep_balance.cu", "asep_resident.cuh", "asep_domain.cuh", "asep_device.cuh", "asep_internal.h"),
-    "sca": ("asep_sca.cu", "asep_device.cuh", "asep_internal.h"),
-    "sca_stream": ("asep_sca.cu", "asep_device.cuh", "asep_internal.h"),
+    "sca": ("asep_sca.cu", "asep_sca.cuh", "asep_device.cuh", "asep_internal.h"),
+    "sca_stream": ("asep_sca.cu", "asep_sca.cuh", "asep_device.cuh", "asep_internal.h"),
     "stream": ("asep_stream.cu", "asep_domain.cuh", "asep_device.cuh", "asep_internal.h"),
     "serial": ("asep_serial.cu", "asep_device.cuh", "asep_internal.h"),
 }
@@ -546,7 +546,7 @@ def batch_mode_table(n_contexts: int = 64, step_sweeps: int = 8, steps: int = 50
 
 def sca_growth(steps: int, peak_ops: float):
     """The benchmarked workload under the paper's own schedule, the
-    two-sub-lattice SCA (k_sca): same rings, rates, sweeps and sample times,
+    two-sub-lattice SCA (k_sca_tile): same rings, rates, sweeps and sample times,
     re-drawn initial state + 2^14 sweeps per step, device-timed."""
     import torch
 
@@ -575,7 +575,7 @@ def sca_growth(steps: int, peak_ops: float):
     achieved = rate * SCA_OPS_PER_ATTEMPT
     return {"workload": "the same growth-regime workload under the paper's two-sub-lattice SCA schedule "
                         "(even bonds, then odd bonds, one attempt per bond per sweep)",
-            "attempts_per_s": rate, "ms_per_step": t, "steps": steps, "kernel": "k_sca",
+            "attempts_per_s": rate, "ms_per_step": t, "steps": steps, "kernel": "k_sca_tile",
             "threads_per_cta": info["threads"],
             "roofline": {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12, "unit": "Tops/s",
                          "frac": achieved / peak_ops, "ops_per_attempt": SCA_OPS_PER_ATTEMPT,
@@ -623,8 +623,8 @@ def window_cases():
          "ASEP p=0.75 q=0.25, 16 samples, 200-MCS window",
          dict(L=1 << 24, domain_sites=256, samples_per_real=16, p_thr=th(0.75), q_thr=th(0.25), seed=1,
               flags=A.ASEP_FLAG_NO_HOP_COUNTS), [200], 1),
-        ("streamed SCA: L=2^28 rings (the paper's one-large-sample-per-GPU mode; lattice in HBM, a thread per "
-         "8 words, one launch per phase), ASEP p=0.75 q=0.25, 8 samples (256 MB, beyond L2), 200-MCS window",
+        ("streamed SCA: L=2^28 rings (the paper's one-large-sample-per-GPU mode; lattice in HBM, a warp per tile, "
+         "up to 128 sweeps a launch), ASEP p=0.75 q=0.25, 8 samples (256 MB, beyond L2), 200-MCS window",
          dict(L=1 << 28, schedule=A.ASEP_SCHED_SCA, samples_per_real=8, p_thr=th(0.75), q_thr=th(0.25), seed=1,
               flags=A.ASEP_FLAG_NO_HOP_COUNTS), [200], 1),
     ]
@@ -678,7 +678,7 @@ def other_workloads(tune: bool = True, peak_ops: float | None = None, rng_bitop:
             attempts = lanes * kw["L"] * info["S"] * n_sweeps
             row = {"workload": name, "attempts": attempts, "ms": ms, "attempts_per_s": attempts / (ms / 1e3),
                    "kernel": ("k_serial" if kw.get("schedule") == A.ASEP_SCHED_SERIAL
-                              else ("k_sca_stream" if info["cluster"] == 32 else "k_sca")
+                              else "k_sca_tile"
                               if kw.get("schedule") == A.ASEP_SCHED_SCA
                               else "k_stream" if info["cluster"] == 32
                               else "k_cluster" if info["cluster"] > 1 else "k_domain"),
@@ -699,9 +699,11 @@ def other_workloads(tune: bool = True, peak_ops: float | None = None, rng_bitop:
                     row["roofline"]["smem_frac"] = sm["frac"]
                     row["roofline"]["smem_wavefronts_per_attempt"] = sm["wavefronts_per_attempt"]
             if info["cluster"] == 32:
-                # streamed: each phase reads and writes every lattice word once (4 x L/8 bytes per plane
-                # and sweep); the whole window, launch gaps and records included, against measured HBM
-                alg = 4 * (kw["L"] // 8) * lanes * info["S"] * n_sweeps
+                # streamed: each phase (the automaton: each launch of up to 128 sweeps) reads and writes every
+                # lattice word once, 2 x L/8 bytes per plane; the whole window, launch gaps and records included,
+                # against measured HBM
+                passes = -(-n_sweeps // 128) if kw.get("schedule") == A.ASEP_SCHED_SCA else 2 * n_sweeps
+                alg = 2 * (kw["L"] // 8) * lanes * info["S"] * passes
                 gbs = alg / (ms / 1e3) / 1e9
                 measured = _peaks().get("hbm_gbs")
                 peak = measured or 6800.0
@@ -768,16 +770,17 @@ def profile_case(schedule: str = "domain"):
                   launch is that of a full step);
     "domain_bal"  the same as a balanced launch (k_domain_bal), 512 sweeps in
                   chunks of 32: the groups move between SMs 16 times;
-    "sca"         the same workload under the two-sub-lattice SCA (k_sca);
-    "sca_stream"  two sweeps (four launches, one per phase) of the streamed
-                  SCA on 8 rings of 2^28 sites (256 MB);
+    "sca"         the same workload under the two-sub-lattice SCA (k_sca_tile);
+    "sca_stream"  128 sweeps (one launch) of the SCA on 8 rings of 2^28 sites
+                  (256 MB);
     "stream"      two sweeps (four launches) of the streamed domain tier
                   (k_stream) on 16 rings of 2^24 sites (32 MB), the bench's
                   streamed window;
     "serial"      1000 sweeps of the serial schedule on the plain-TASEP
                   configuration (L = 4096, 8 samples; its automatic plan, one
-                  CTA per sample running each sweep in dependency rounds);
-    "window<i>"   window i of window_cases(), 32 sweeps (streamed: 2);
+                  CTA per sample);
+    "window<i>"   window i of window_cases(), 32 sweeps (streamed: 2; long
+                  automaton rings: 128);
     "attempt_bench" the RNG + bit-op microbenchmark at full occupancy
                   (152 x 8 CTAs of 256 threads, 4096 Philox calls each), the
                   measured roof of the domain schedule."""
@@ -795,10 +798,10 @@ def profile_case(schedule: str = "domain"):
               flush=True)
         return 0
     if schedule.startswith("window"):
-        # one window of the other configurations, briefly: 32 sweeps (streamed ones 2), one record at the end
+        # one window of the other configurations, briefly: 32 sweeps (see above), one record at the end
         name, kw, times, lanes = window_cases()[int(schedule[len("window"):])]
         kw = dict(kw)
-        n = 2 if kw["L"] >= 1 << 24 else 32
+        n = 32 if kw["L"] < 1 << 24 else 128 if kw.get("schedule") == A.ASEP_SCHED_SCA else 2
         if kw.get("flags", 0) & A.ASEP_FLAG_AUTOCORR:
             kw["autocorr_t0"] = n
         with A.asep_create(A.make_params(**kw), sample_times=[n]) as ctx:
@@ -812,7 +815,7 @@ def profile_case(schedule: str = "domain"):
         if schedule == "sca_stream":
             prm = A.make_params(L=1 << 28, schedule=A.ASEP_SCHED_SCA, samples_per_real=8, p_thr=th(P_RATE),
                                 q_thr=th(Q_RATE), seed=SEED, flags=A.ASEP_FLAG_NO_HOP_COUNTS)
-            n = 2
+            n = 128
         elif schedule == "stream":
             prm = A.make_params(L=1 << 24, domain_sites=256, samples_per_real=16, p_thr=th(P_RATE), q_thr=th(Q_RATE),
                                 seed=SEED, flags=A.ASEP_FLAG_NO_HOP_COUNTS)

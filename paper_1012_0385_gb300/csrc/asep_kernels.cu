@@ -13,7 +13,7 @@
 //               turning sites (paper sec. 3), one bit per site.
 //   k_domain    the resident two-phase Poisson-domain sweep: a CTA holds one
 //               or more whole rings in shared memory for a whole launch.
-//   (k_serial, the exact serial schedule, is in asep_serial.cu; k_sca, the
+//   (k_serial, the exact serial schedule, is in asep_serial.cu; k_sca_tile, the
 //   paper's two-sub-lattice schedule, in asep_sca.cu.)
 //   k_heights   h_i = sum_{j<=i} (2 n_j - 1) and the sums of Eq. (W)
 //               (k_heights_part + k_heights_combine for long lattices).

@@ -12,13 +12,13 @@
 namespace asep {
 
 // Plans of the serial schedule (asep_info.cluster of a serial context).
-constexpr uint32_t kSerialRounds = 1;  // one CTA per sample, the sweep's attempts in dependency rounds
-constexpr uint32_t kSerialWarp = 2;    // one warp per sample, committed prefixes of up to 32 attempts
-constexpr uint32_t kSerialRoundsMaxAttempts = 32u * 1024u;  // attempts per sweep: 32 per thread of a CTA
+constexpr uint32_t kSerialRounds = 1;  // one CTA per sample
+constexpr uint32_t kSerialWarp = 2;    // one warp per sample
+constexpr uint32_t kSerialRoundsMaxAttempts = 32u * 1024u;  // attempts per sweep
 constexpr size_t kSerialRoundsSmem = 200u * 1024u;
 
 // Dynamic shared memory of the one-CTA plan (lattice, quenched planes, site
-// table, the sweep's draws), or 0 when the plan does not apply to L.
+// tables, ring of drawn attempts), or 0 when the plan does not apply to L.
 size_t serial_rounds_smem_bytes(uint32_t model, uint32_t dis, uint64_t L);
 // Threads per CTA of the one-CTA plan.
 uint32_t serial_rounds_threads(uint32_t model, uint64_t L);
