@@ -275,19 +275,21 @@ __global__ void __launch_bounds__(1024, 1) k_cluster(const DomainLaunch a) {
 
 }  // namespace
 
+// The kernel's limits, the same whatever a launch needs: contexts of several
+// threads launch it side by side, and none may lower what another has set.
 template <uint32_t MODEL, uint32_t DIS, bool COUNT>
-cudaError_t cluster_attrs(uint32_t cluster, size_t smem) {
-  cudaError_t e = cudaFuncSetAttribute(k_cluster<MODEL, DIS, COUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e == cudaSuccess && cluster > 8)
-    e = cudaFuncSetAttribute(k_cluster<MODEL, DIS, COUNT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  return e;
+cudaError_t cluster_attrs() {
+  const cudaError_t e = cudaFuncSetAttribute(k_cluster<MODEL, DIS, COUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             227 * 1024 - 64);
+  return e != cudaSuccess
+             ? e
+             : cudaFuncSetAttribute(k_cluster<MODEL, DIS, COUNT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 
 template <uint32_t MODEL, uint32_t DIS, bool COUNT>
 cudaError_t launch_cluster_t(const DomainLaunch& a, uint32_t threads, size_t smem, cudaStream_t st) {
   (void)cudaGetLastError();
-  cudaError_t e = cluster_attrs<MODEL, DIS, COUNT>(a.cluster, smem);
+  const cudaError_t e = cluster_attrs<MODEL, DIS, COUNT>();
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(a.geo.S * a.cluster, 1, 1);
@@ -306,7 +308,7 @@ cudaError_t launch_cluster_t(const DomainLaunch& a, uint32_t threads, size_t sme
 
 template <uint32_t MODEL, uint32_t DIS, bool COUNT>
 int cluster_fits_t(uint32_t cluster, uint32_t threads, size_t smem) {
-  if (cluster_attrs<MODEL, DIS, COUNT>(cluster, smem) != cudaSuccess) {
+  if (cluster_attrs<MODEL, DIS, COUNT>() != cudaSuccess) {
     (void)cudaGetLastError();
     return 0;
   }
