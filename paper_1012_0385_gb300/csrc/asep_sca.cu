@@ -41,6 +41,17 @@ constexpr uint32_t kScaTileSweeps = 128;  // sweeps a launch: the halo's 256 sit
 // rings of 2^20 (20824) 6.96 / 6.80, 8 rings of 2^28 90.3 / 86.9.
 constexpr uint64_t kScaManyTiles = 152u * 108u;
 
+// Kinds without a fixed number of planes: a phase of a warp lasts until the
+// last of its candidates is decided (some log2 of their number planes), or its
+// queue of lane changes is done, so where the tiles are fewer than the
+// schedulers, rings are cut into smaller ones, of four units at least, while
+// no scheduler has two.  us per sweep without and with: 76 rings of 32 units with
+// slow classes 3.50 -> 3.14, 113 of 19 units 3.30 -> 2.95, 191 pairs of lanes of
+// 25 units with turning sites 5.29 -> 3.98; cut further, to two warps a scheduler,
+// 265 rings of 14 units 3.17 -> 3.95.
+constexpr uint64_t kScaFewTiles = 4u * 152u;
+constexpr uint32_t kScaFewUnits = 4u;
+
 // One launch of k_sca_tile.
 struct ScaTileLaunch {
   uint32_t tiles, units;  // per ring: tiles, units per tile (the last may hold fewer)
@@ -71,7 +82,7 @@ struct ScaTileLaunch {
 // one CTA per ring with two barriers a sweep, and against one launch per phase
 // with the lattice streamed through HBM, us per sweep: 256 rings of 2^17 at
 // p = 0.75, q = 0.25 1.90 -> 1.65, 201 rings of 391 units with independent
-// classes 13.0 -> 8.6, 128 pairs of lanes of 2^16 with turning sites 6.35 ->
+// classes 13.0 -> 9.0, 128 pairs of lanes of 2^16 with turning sites 6.35 ->
 // 6.5, 2 rings of 2^22 10.3 -> 0.60, 8 rings of 2^28 189 -> 87.
 //
 // Records are taken inside the launch: a tile leaves the sums of its heights
@@ -471,8 +482,7 @@ size_t sca_smem_bytes(uint32_t W, uint32_t planes, uint32_t quenched_planes) {
 
 ScaTiles sca_tiles(uint32_t model, uint32_t dis, uint32_t p_thr, uint32_t q_thr, uint32_t W, uint32_t S) {
   const uint32_t n = W / 8u;
-  const auto cut = [n](uint32_t upt) {
-    const uint32_t most = 32u * upt - 2u;
+  const auto cut = [n](uint32_t upt, uint32_t most) {
     ScaTiles t;
     t.upt = upt;
     t.tiles = (n + most - 1u) / most;
@@ -480,9 +490,16 @@ ScaTiles sca_tiles(uint32_t model, uint32_t dis, uint32_t p_thr, uint32_t q_thr,
     t.tiles = (n + t.units - 1u) / t.units;
     return t;
   };
-  const ScaTiles one = cut(1);
-  if (model != kRing || dis != kDisNone || sca_fast(p_thr, q_thr) == kScaAny) return one;
-  return static_cast<uint64_t>(one.tiles) * S <= kScaManyTiles ? one : cut(2);
+  const ScaTiles one = cut(1, 30u);
+  if (model == kRing && dis == kDisNone && sca_fast(p_thr, q_thr) != kScaAny)
+    return static_cast<uint64_t>(one.tiles) * S <= kScaManyTiles ? one : cut(2, 62u);
+  // kinds whose warps run to their most undecided bond (or longest queue of lane changes)
+  ScaTiles best = one;
+  for (uint32_t u = 29u; u >= kScaFewUnits; --u) {
+    const ScaTiles t = cut(1, u);
+    if (static_cast<uint64_t>(t.tiles) * S <= kScaFewTiles) best = t;
+  }
+  return best;
 }
 
 size_t sca_halo_words(const ScaTiles& t, uint32_t S, uint32_t planes) {

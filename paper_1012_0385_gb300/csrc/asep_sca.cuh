@@ -164,53 +164,25 @@ __device__ __forceinline__ ScaRule sca_rule(const Rates& r, bool dis) {
 
 constexpr uint32_t kScaBlock = 7;  // planes taken without looking for undecided lanes
 
-// One plane of the comparison from the least significant side: lt = u < t and
-// eq = u == t over the planes so far; the threshold bit is b1 where z is set,
-// b0 elsewhere (uniform).
-__device__ __forceinline__ void compare_up(const uint32_t (&z)[4], bool b1, bool b0, const uint4 y, uint32_t (&lt)[4],
-                                           uint32_t (&eq)[4]) {
-  const uint32_t u[4] = {y.x, y.y, y.z, y.w};
-  if (b1 == b0) {
-    if (b1) {
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        lt[g] |= ~u[g];
-        eq[g] &= u[g];
-      }
-    } else {
-#pragma unroll
-      for (int g = 0; g < 4; ++g) {
-        lt[g] &= ~u[g];
-        eq[g] &= ~u[g];
-      }
-    }
-  } else if (b1) {
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      lt[g] = bitsel(z[g], lt[g] | ~u[g], lt[g] & ~u[g]);
-      eq[g] &= ~(z[g] ^ u[g]);
-    }
-  } else {
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      lt[g] = bitsel(z[g], lt[g] & ~u[g], lt[g] | ~u[g]);
-      eq[g] &= z[g] ^ u[g];
-    }
-  }
-}
-
 // Any thresholds.  c1: slow classes of the first sites (right hops), c2: of
 // the second sites (left hops); DIS = false: no classes.  The first kScaBlock
 // planes decide all but a few of a warp's some 2000 candidates, so they are
-// compared from the least significant side (two logic operations a group and
-// plane, no vote); the rest most significant first, until no candidate of the
-// warp is undecided (some 12 planes in all).  All 32 lanes call.
+// compared from the least significant side (lt = u < t and eq = u == t over the
+// planes so far, no vote); the rest most significant first, until no candidate
+// of the warp is undecided (some 12 planes in all).  All 32 lanes call.
+// Without branches inside a plane: asking whether the thresholds' bits agree
+// saves a logic operation a group there (rings of 2^17 at p = 0.8, q = 0.2 14.4
+// us a sweep instead of 14.6, 201 rings of 391 units with four classes 8.74
+// instead of 9.0), but where a scheduler has one warp, each branch is a wait:
+// 76 rings of 32 units with classes 3.14 -> 2.66, 265 of 14 units 3.17 -> 2.86
+// (both with the smaller tiles).  Two calls in flight: no gain there, 3-5 %
+// slower with classes.
 template <bool DIS, typename PLANE>
 __device__ __forceinline__ void decide_any(const uint32_t (&f)[4], const uint32_t (&n)[4], const uint32_t (&c1)[4],
                                            const uint32_t (&c2)[4], const Rates& r, const ScaRule& rule, uint32_t kmax,
                                            PLANE plane, uint32_t (&h)[4]) {
   constexpr uint32_t kAll = 0xFFFFFFFFu;
-  uint32_t eq[4], cand[4], sl[4], z[4];
+  uint32_t eq[4], cand[4], sl[4];
 #pragma unroll
   for (int g = 0; g < 4; ++g) {
     cand[g] = f[g] ^ n[g];
@@ -231,51 +203,52 @@ __device__ __forceinline__ void decide_any(const uint32_t (&f)[4], const uint32_
     }
   }
   const uint32_t kb = min(kmax, kScaBlock);
-  const bool two = !DIS || rule.by_class;  // one selector tells the planes apart
 #pragma unroll
-  for (int g = 0; g < 4; ++g) {
-    z[g] = DIS ? sl[g] : f[g];
-    eq[g] = cand[g];
-  }
-  if (kb) {
+  for (int g = 0; g < 4; ++g) eq[g] = cand[g];
+  // bit k of every lane's threshold: one selector tells two thresholds apart (no classes: the first sites; classes
+  // that right and left hops share: the classes), or classes and first sites four
+  const auto two = [&](uint32_t k, uint32_t (&t)[4]) {
+    const uint32_t m1 = bit_mask(DIS ? rule.ps : rule.p, k), m0 = bit_mask(DIS ? rule.p : rule.q, k);
+#pragma unroll
+    for (int g = 0; g < 4; ++g) t[g] = bitsel(DIS ? sl[g] : f[g], m1, m0);
+  };
+  const auto four = [&](uint32_t k, uint32_t (&t)[4]) {
+    const uint32_t mp = bit_mask(rule.p, k), mq = bit_mask(rule.q, k), mps = bit_mask(rule.ps, k), mqs = bit_mask(rule.qs, k);
+#pragma unroll
+    for (int g = 0; g < 4; ++g) t[g] = bitsel(f[g], bitsel(sl[g], mps, mp), bitsel(sl[g], mqs, mq));
+  };
+  const auto run = [&](auto bits) {
     uint32_t lt[4] = {0u, 0u, 0u, 0u};
-#pragma unroll 1
-    for (uint32_t k = kb; k-- > 0;) {
-      const uint4 y = plane(k);
-      const uint32_t sh = 19u - k;
-      const bool P = (rule.p >> sh) & 1u, Q = (rule.q >> sh) & 1u, PS = (rule.ps >> sh) & 1u, QS = (rule.qs >> sh) & 1u;
-      if (two) {
-        compare_up(z, DIS ? PS : P, DIS ? P : Q, y, lt, eq);
-      } else {
-        const uint32_t u[4] = {y.x, y.y, y.z, y.w};
-        const uint32_t mp = P ? ~0u : 0u, mq = Q ? ~0u : 0u, mps = PS ? ~0u : 0u, mqs = QS ? ~0u : 0u;
+    const auto up = [&](uint32_t k, const uint4 y) {
+      const uint32_t u[4] = {y.x, y.y, y.z, y.w};
+      uint32_t t[4];
+      bits(k, t);
 #pragma unroll
-        for (int g = 0; g < 4; ++g) {
-          const uint32_t t = bitsel(f[g], bitsel(sl[g], mps, mp), bitsel(sl[g], mqs, mq));
-          lt[g] = bitsel(t, lt[g] | ~u[g], lt[g] & ~u[g]);
-          eq[g] &= ~(t ^ u[g]);
-        }
+      for (int g = 0; g < 4; ++g) {
+        lt[g] = bitsel(t[g], lt[g] | ~u[g], lt[g] & ~u[g]);
+        eq[g] &= ~(t[g] ^ u[g]);
       }
-    }
+    };
+#pragma unroll 1
+    for (uint32_t k = kb; k-- > 0;) up(k, plane(k));
 #pragma unroll
     for (int g = 0; g < 4; ++g) h[g] |= cand[g] & lt[g];
-  }
 #pragma unroll 1
-  for (uint32_t k = kb; k < kmax; ++k) {
-    if (!__any_sync(0xffffffffu, (eq[0] | eq[1] | eq[2] | eq[3]) != 0u)) break;
-    const uint4 y = plane(k);
-    const uint32_t u[4] = {y.x, y.y, y.z, y.w};
-    const uint32_t P = bit_mask(rule.p, k), Q = bit_mask(rule.q, k);
-    const uint32_t PS = DIS ? bit_mask(rule.ps, k) : 0u, QS = DIS ? bit_mask(rule.qs, k) : 0u;
+    for (uint32_t k = kb; k < kmax; ++k) {
+      if (!__any_sync(0xffffffffu, (eq[0] | eq[1] | eq[2] | eq[3]) != 0u)) break;
+      const uint4 y = plane(k);
+      const uint32_t u[4] = {y.x, y.y, y.z, y.w};
+      uint32_t t[4];
+      bits(k, t);
 #pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      const uint32_t t = !DIS ? bitsel(f[g], P, Q)
-                         : rule.by_class ? bitsel(sl[g], PS, P)
-                                         : bitsel(f[g], bitsel(sl[g], PS, P), bitsel(sl[g], QS, Q));
-      h[g] |= eq[g] & t & ~u[g];  // this bit of u is 0 where t's is 1: u < t
-      eq[g] &= ~(t ^ u[g]);       // equal so far
+      for (int g = 0; g < 4; ++g) {
+        h[g] |= eq[g] & t[g] & ~u[g];  // this bit of u is 0 where t's is 1: u < t
+        eq[g] &= ~(t[g] ^ u[g]);       // equal so far
+      }
     }
-  }
+  };
+  if (!DIS || rule.by_class) run(two);
+  else run(four);
 }
 
 // In-lane bonds of one lane of the two-lane model: candidates cand, one

@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(256) k_serial(const SerialLaunch a, uint32_t h
 // scheduler) and its chain of shared-memory steps: some 950 clocks.  Measured
 // against rounds over a whole sweep, whose attempts were visited 2.5 times at
 // two barriers a round, us per sweep of 8 rings of 4096: 14.7 -> 4.85 (a window
-// of 256 6.9, of 512 in two attempts a thread 6.6, 1024 threads 6.4).
+// of 256 6.9, of 512 in two attempts a thread 6.6).
 
 // Sums over the block (all threads call): a signed 64-bit value and an
 // unsigned 64-bit value summed exactly in 128 bits.  Results valid in thread 0.
