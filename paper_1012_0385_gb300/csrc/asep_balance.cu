@@ -115,11 +115,16 @@ cudaError_t launch_bal_cp(const DomainLaunch& a, const BalanceLaunch& b, uint32_
       (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
     return e;
   if (per_sm <= 0) return cudaErrorInvalidConfiguration;
-  // As many slots per SM as the groups need (ceil(groups / SMs)), not as many
-  // as fit: with more, groups that migrate would pile onto some SMs while
-  // others empty.  The slots beyond the groups float between SMs.
+  // Slots per SM: as near to 17 warps as whole CTAs come, and no more than the
+  // groups need (ceil(groups / SMs)).  Some four warps a scheduler fill the
+  // pipes; with more slots, groups pile onto some SMs while others empty, and
+  // every chunk waits for its slowest predecessor.  us per sweep with 1 / 2 / 3
+  // slots: 256 groups of 8 warps 55 / 46 / 53, 400 of 8 88 / 64 / 71, 400 of 4
+  // 81 / 48 / 42 (4: 45), 500 of 7 130 / 85 / 89, 361 of 11 111 / 94 / 121, 200
+  // of 15 71 / 95 / 99, 361 of 20 152 / 178 / 176.
   const uint32_t need = (a.n_groups + static_cast<uint32_t>(sms) - 1) / static_cast<uint32_t>(sms);
-  const uint32_t slots = std::min<uint32_t>(static_cast<uint32_t>(per_sm), need);
+  const uint32_t warps = (threads + 31u) / 32u, fill = std::max<uint32_t>(1, (2u * 17u + warps) / (2u * warps));
+  const uint32_t slots = std::min<uint32_t>(static_cast<uint32_t>(per_sm), std::min(need, fill));
   const uint32_t items = a.n_groups * b.chunks;
   const uint32_t ctas = std::max<uint32_t>(1, std::min<uint32_t>(items, slots * static_cast<uint32_t>(sms)));
   if ((e = cudaMemsetAsync(b.progress, 0, (a.n_groups + 1u) * sizeof(uint32_t), st)) != cudaSuccess) return e;
