@@ -396,7 +396,10 @@ int asep_batch_create(void* stream, uint32_t max_jobs, uint32_t max_items, asep_
 int asep_batch_sweep(asep_batch* b, asep_ctx* const* ctxs, const uint64_t* n_mcs, uint32_t n);
 
 /* Capture one batch step (these contexts, these sweep counts) as a CUDA
- * graph on the first call for this set, then launch it `replays` times.
+ * graph on the first call for this set, then launch it `replays` times.  A
+ * later call with the same contexts and sweeps launches the same graph; one
+ * with others, or after asep_reset or asep_set_plan of one of them, captures
+ * its own.  Other steps of the batch may run between the calls.
  * The sweep index and the sample-time cursor of each context live in device
  * memory and advance with every replay.  Asynchronous. */
 int asep_batch_graph(asep_batch* b, asep_ctx* const* ctxs, const uint64_t* n_mcs, uint32_t n, uint32_t replays);

@@ -8,6 +8,7 @@
 // per-lane 32-bit hop counters cannot wrap, and tells each launch which of
 // its sweep counts are sample times.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -25,6 +26,9 @@
 using namespace asep;
 
 struct asep_ctx {
+  // which context a captured step holds, and in which state: addresses are used again once a context is destroyed
+  uint64_t id = 0;          // of no other context of the process
+  uint64_t generation = 0;  // moved on by whatever changes a launch's descriptor (seed, plan)
   asep_params p{};
   uint64_t L = 0;
   uint32_t D = 0, logD = 0, planes = 1, W = 0, S = 0, R = 0;
@@ -838,6 +842,8 @@ int asep_create(const asep_params* params, asep_ctx** out) {
   if (rc != ASEP_OK) return rc;
   asep_ctx* ctx = new (std::nothrow) asep_ctx();
   if (!ctx) return fail(nullptr, ASEP_ERR_NOMEM, "host allocation failed");
+  static std::atomic<uint64_t> last_id{0};
+  ctx->id = ++last_id;
 
   auto bail = [&](int code) {
     g_create_error = ctx->err;
@@ -1023,6 +1029,7 @@ int asep_reset(asep_ctx* ctx, uint64_t seed, uint64_t init_seed) {
   if (!ctx) return ASEP_ERR_INVALID;
   const int rct = clear_timeout(ctx);  // a new initial state replaces results a timed-out sweep invalidated
   if (rct != ASEP_OK) return rct;
+  ++ctx->generation;
   ctx->p.seed = seed;
   ctx->p.init_seed = init_seed;
   const size_t n_times = std::max<size_t>(1, ctx->times.size());
@@ -1193,7 +1200,8 @@ struct asep_batch {
   cudaEvent_t fork = nullptr, join[kAuxStreams] = {};
   // graph cache: one captured step
   cudaGraphExec_t exec = nullptr;
-  std::vector<uintptr_t> graph_key;
+  std::vector<uint64_t> graph_key;  // per context: id, generation, sweeps
+  bool graph_live = false;          // d_jobs and d_items hold what the captured step reads
   std::string err;
 };
 
@@ -1234,6 +1242,7 @@ int batch_prepare(asep_batch* b, asep_ctx* const* ctxs, const uint32_t* n, uint3
     uint32_t code;
   };
   std::vector<It> items;
+  b->graph_live = false;  // the caller's step takes the place of a captured one's
   cudaError_t e = cudaEventSynchronize(b->staged);
   if (e != cudaSuccess) return bfail(b, ASEP_ERR_CUDA, "staging event: %s", cudaGetErrorString(e));
   for (uint32_t j = 0; j < nj; ++j) {
@@ -1463,25 +1472,28 @@ int asep_batch_graph(asep_batch* b, asep_ctx* const* ctxs, const uint64_t* n_mcs
   int rc = batch_check(b, ctxs, n_mcs, n);
   if (rc != ASEP_OK || n == 0 || replays == 0) return rc;
   std::vector<uint32_t> step(n);
-  std::vector<uintptr_t> key;
+  std::vector<uint64_t> key;
   for (uint32_t j = 0; j < n; ++j) {
     if (n_mcs[j] > sweeps_cap(ctxs[j]))
       return bfail(b, ASEP_ERR_INVALID, "context %u: a graph step is at most one launch of sweeps", j);
     step[j] = static_cast<uint32_t>(n_mcs[j]);
-    key.push_back(reinterpret_cast<uintptr_t>(ctxs[j]));
-    key.push_back(step[j]);
+    key.insert(key.end(), {ctxs[j]->id, ctxs[j]->generation, step[j]});
   }
   if ((rc = order_in(b, ctxs, n)) != ASEP_OK) return rc;
   cudaError_t e;
-  if (!b->exec || key != b->graph_key) {
+  // Descriptors and items are uploaded outside the graph: once, and again where another step of this batch has
+  // uploaded its own since.
+  uint32_t n_items = 0, threads = 0, ctas = 0;
+  size_t smem = 0;
+  const bool captured = b->exec && key == b->graph_key;
+  if (!captured || !b->graph_live) {
+    if ((rc = batch_prepare(b, ctxs, step.data(), n, &n_items, &threads, &ctas, &smem)) != ASEP_OK) return rc;
+  }
+  if (!captured) {
     if (b->exec) {
       cudaGraphExecDestroy(b->exec);
       b->exec = nullptr;
     }
-    uint32_t n_items, threads, ctas;
-    size_t smem;
-    // descriptors and items are uploaded once, outside the graph
-    if ((rc = batch_prepare(b, ctxs, step.data(), n, &n_items, &threads, &ctas, &smem)) != ASEP_OK) return rc;
     // kernel attributes are set before capture begins
     if (batch_ctas_per_sm(threads, smem) <= 0) return bfail(b, ASEP_ERR_INVALID, "batch kernel does not fit");
     // capture on the batch's own stream (nothing runs during capture), launch on b->stream
@@ -1503,6 +1515,7 @@ int asep_batch_graph(asep_batch* b, asep_ctx* const* ctxs, const uint64_t* n_mcs
     }
     b->graph_key = key;
   }
+  b->graph_live = true;
   for (uint32_t r = 0; r < replays; ++r) {
     if ((e = cudaGraphLaunch(b->exec, b->stream)) != cudaSuccess)
       return bfail(b, ASEP_ERR_CUDA, "graph launch: %s", cudaGetErrorString(e));
@@ -1542,6 +1555,7 @@ const char* asep_batch_last_error(const asep_batch* b) { return b ? b->err.c_str
 
 int asep_set_plan(asep_ctx* ctx, uint32_t cluster, uint32_t samples_per_group) {
   if (!ctx) return ASEP_ERR_INVALID;
+  ++ctx->generation;
   if (ctx->p.schedule == ASEP_SCHED_SCA) {
     if (cluster > 1 && cluster != kStreamTier)
       return fail(ctx, ASEP_ERR_INVALID, "SCA plans: cluster 0 (choose), 1 (resident) or 32 (streamed)");
