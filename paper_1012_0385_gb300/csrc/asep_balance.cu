@@ -104,8 +104,7 @@ template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP>
 cudaError_t launch_bal_cp(const DomainLaunch& a, const BalanceLaunch& b, uint32_t threads, size_t smem,
                           cudaStream_t st) {
   (void)cudaGetLastError();
-  cudaError_t e = cudaFuncSetAttribute(k_domain_bal<MODEL, DIS, COUNT, CP>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  cudaError_t e = allow_smem(k_domain_bal<MODEL, DIS, COUNT, CP>, kSmemOptIn - 16);  // 16: s_item, s_ok
   if (e != cudaSuccess) return e;
   int per_sm = 0, dev = 0, sms = 0;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_domain_bal<MODEL, DIS, COUNT, CP>,

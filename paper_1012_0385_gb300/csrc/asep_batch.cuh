@@ -64,14 +64,14 @@ __global__ void __maxnreg__(MAXT == 512 ? 104 : 64) k_batch(const DomainLaunch* 
 // shared memory -- the item index and the descriptor copy -- counts against
 // the same limit), launch, occupancy.
 template <uint32_t MAXT>
-cudaError_t batch_attr(size_t smem) {
-  return cudaFuncSetAttribute(k_batch<MAXT>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+cudaError_t batch_attr() {
+  return allow_smem(k_batch<MAXT>, kSmemOptIn - sizeof(DomainLaunch) - 64);
 }
 
 template <uint32_t MAXT>
 cudaError_t batch_launch(const DomainLaunch* jobs, const uint32_t* items, uint32_t n_items, uint32_t* queue,
                          uint32_t threads, uint32_t ctas, size_t smem, cudaStream_t st) {
-  const cudaError_t e = batch_attr<MAXT>(smem);
+  const cudaError_t e = batch_attr<MAXT>();
   if (e != cudaSuccess) return e;
   k_batch<MAXT><<<ctas, threads, smem, st>>>(jobs, items, n_items, queue);
   return cudaGetLastError();
@@ -79,7 +79,7 @@ cudaError_t batch_launch(const DomainLaunch* jobs, const uint32_t* items, uint32
 
 template <uint32_t MAXT>
 cudaError_t batch_occupancy(uint32_t threads, size_t smem, int* n) {
-  const cudaError_t e = batch_attr<MAXT>(smem);
+  const cudaError_t e = batch_attr<MAXT>();
   return e != cudaSuccess ? e
                           : cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_batch<MAXT>, static_cast<int>(threads), smem);
 }

@@ -275,12 +275,10 @@ __global__ void __launch_bounds__(1024, 1) k_cluster(const DomainLaunch a) {
 
 }  // namespace
 
-// The kernel's limits, the same whatever a launch needs: contexts of several
-// threads launch it side by side, and none may lower what another has set.
+// The kernel's limits, the same whatever a launch needs (allow_smem).
 template <uint32_t MODEL, uint32_t DIS, bool COUNT>
 cudaError_t cluster_attrs() {
-  const cudaError_t e = cudaFuncSetAttribute(k_cluster<MODEL, DIS, COUNT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             227 * 1024 - 64);
+  const cudaError_t e = allow_smem(k_cluster<MODEL, DIS, COUNT>, kSmemOptIn - 64);  // 64: cta_sums
   return e != cudaSuccess
              ? e
              : cudaFuncSetAttribute(k_cluster<MODEL, DIS, COUNT>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);

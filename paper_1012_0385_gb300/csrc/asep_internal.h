@@ -211,6 +211,16 @@ cudaError_t launch_domain_balanced(const DomainLaunch& a, const BalanceLaunch& b
 
 // Shared memory of the resident kernel, in bytes (planes of R2 + 1 rows:
 // the extra row mirrors the next column's row 0).
+// Dynamic shared memory a kernel may be launched with: `most` is the same for
+// every launch of a kernel, never what one launch needs.  Contexts of several
+// host threads launch a kernel side by side, and a limit set for a small
+// context between another thread's call here and its launch would refuse that
+// launch.
+constexpr size_t kSmemOptIn = 227 * 1024;  // static and dynamic, per CTA
+template <typename K>
+inline cudaError_t allow_smem(K* kernel, size_t most) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+}
 size_t domain_smem_bytes(uint32_t model, uint32_t dis, uint32_t R2, uint32_t Cp, uint32_t ptab_n, uint32_t threads);
 
 cudaError_t launch_init(const InitLaunch& a, cudaStream_t st);

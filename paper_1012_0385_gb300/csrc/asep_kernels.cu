@@ -252,10 +252,9 @@ __global__ void k_advance_batch(const DomainLaunch* jobs, uint32_t n_jobs) {
 
 template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t CP>
 cudaError_t launch_domain_cp(const DomainLaunch& a, uint32_t threads, size_t smem, cudaStream_t st) {
-  // set per call to what this launch needs: cheap, and right on every device
+  // set on every call: cheap, and right on every device
   (void)cudaGetLastError();
-  const cudaError_t e = cudaFuncSetAttribute(k_domain<MODEL, DIS, COUNT, CP>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = allow_smem(k_domain<MODEL, DIS, COUNT, CP>, kSmemOptIn);
   if (e != cudaSuccess) return e;
   k_domain<MODEL, DIS, COUNT, CP><<<a.n_groups, threads, smem, st>>>(a);
   return cudaGetLastError();

@@ -652,7 +652,7 @@ cudaError_t launch_serial_t(const SerialLaunch& a, cudaStream_t st) {
   const uint32_t blocks = (a.geo.S + warps - 1) / warps;
   const size_t smem = (staged ? per_sample : serial_warp_scratch(hash)) * warps;
   const auto kernel = staged ? k_serial<MODEL, DIS, true> : k_serial<MODEL, DIS, false>;
-  const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = allow_smem(kernel, budget);
   if (e != cudaSuccess) return e;
   kernel<<<blocks, 32 * warps, smem, st>>>(a, hash);
   return cudaGetLastError();
@@ -664,8 +664,7 @@ cudaError_t launch_serial_rounds_t(const SerialLaunch& a, cudaStream_t st) {
   const uint32_t threads = serial_rounds_threads(MODEL, a.geo.L);
   if (smem == 0) return cudaErrorInvalidValue;
   (void)cudaGetLastError();
-  const cudaError_t e = cudaFuncSetAttribute(k_serial_rounds<MODEL, DIS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(smem));
+  const cudaError_t e = allow_smem(k_serial_rounds<MODEL, DIS>, kSerialRoundsSmem);
   if (e != cudaSuccess) return e;
   k_serial_rounds<MODEL, DIS><<<a.geo.S, threads, smem, st>>>(a);
   return cudaGetLastError();

@@ -280,8 +280,7 @@ template <uint32_t MODEL, uint32_t DIS, bool COUNT, uint32_t PHASE>
 cudaError_t launch_stream_t(const DomainLaunch& a, uint32_t tiles, uint32_t threads, size_t smem, uint32_t* err,
                             uint32_t stall, cudaStream_t st) {
   (void)cudaGetLastError();
-  const cudaError_t e = cudaFuncSetAttribute(k_stream<MODEL, DIS, COUNT, PHASE>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const cudaError_t e = allow_smem(k_stream<MODEL, DIS, COUNT, PHASE>, kSmemOptIn - 64);  // 64: its barrier
   if (e != cudaSuccess) return e;
   k_stream<MODEL, DIS, COUNT, PHASE><<<tiles * a.geo.S, threads, smem, st>>>(a, tiles, err, stall);
   return cudaGetLastError();
