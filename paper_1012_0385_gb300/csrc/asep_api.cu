@@ -80,6 +80,7 @@ struct asep_ctx {
   uint32_t* d_halo = nullptr;      // SCA: the tiles' edge units, two halves
   uint32_t sca_records = 0;        // SCA: records a launch holds at most
   ScaPart* d_sca_parts = nullptr;  // SCA: the tiles' parts of a launch's records
+  bool replayed = false;           // asep_sweep was captured into a caller's graph: the device clock alone is right
   uint32_t* d_progress = nullptr;  // balanced launches: [S + 1] chunk flags and queue counter
   uint64_t launches = 0;
   std::string err;
@@ -574,6 +575,16 @@ int record_now(asep_ctx* ctx, uint32_t slot) {
   return ASEP_OK;
 }
 
+// Whether work on the stream is being captured into a graph of the caller's.
+bool is_capturing(cudaStream_t stream) {
+  cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(stream, &status) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return false;
+  }
+  return status != cudaStreamCaptureStatusNone;
+}
+
 // A launch of n sweeps; spread: by the cluster plan ctx->spread.
 DomainLaunch domain_desc(const asep_ctx* ctx, uint32_t n, bool spread = false) {
   DomainLaunch a{};
@@ -968,7 +979,10 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
     } else if (ctx->p.schedule == ASEP_SCHED_DOMAIN && ctx->cluster > 1) {
       e = launch_cluster(domain_desc(ctx, static_cast<uint32_t>(n)), ctx->threads, ctx->smem, ctx->stream);
     } else if (ctx->p.schedule == ASEP_SCHED_SCA) {
+      const bool capturing = is_capturing(ctx->stream);
+      ctx->replayed = ctx->replayed || capturing;
       ScaRun run;
+      run.replayed = capturing || (ctx->replayed && ctx->next_time < ctx->times.size());
       run.halo = ctx->d_halo;
       run.parts = ctx->d_sca_parts;
       run.max_records = ctx->sca_records;

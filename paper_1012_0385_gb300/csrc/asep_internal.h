@@ -276,6 +276,7 @@ struct ScaRun {
   uint64_t sweep;          // sweep count at the start of the call
   const uint64_t* times;   // the sample times not yet recorded
   size_t n_times;
+  bool replayed;           // the launches may run at other sweeps than the host's (captured into a caller's graph)
 };
 // a.n_sweeps sweeps in launches of at most 128, with the records inside them;
 // *launches is advanced.

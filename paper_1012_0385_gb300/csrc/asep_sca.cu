@@ -57,6 +57,7 @@ struct ScaTileLaunch {
   uint32_t tiles, units;  // per ring: tiles, units per tile (the last may hold fewer)
   uint32_t n, offset;     // sweeps of this launch, and before it since the context clock
   uint32_t n_rec, rec_offset;  // sample times inside this launch, and before it since the clock's cursor
+                               // (kScaReplayed: the device finds them, at most n_rec)
   const uint32_t* halo_in;   // [S][tiles][first, last unit][planes][8]
   uint32_t* halo_out;
   ScaPart* parts;         // [n_rec + 1][S][tiles][planes] (the last entry: the launch's hops)
@@ -91,6 +92,29 @@ struct ScaTileLaunch {
 // between launches -- the launch, k_heights, the clock, the next launch --
 // took some 25 us; 256 rings of 2^17 with 88 log-spaced records in 2048
 // sweeps spent 2.2 of 5.6 ms there.)
+
+// Sample times of a launch from sweep s0 on: index of the first, and how many.
+// The host knows both, except of a launch that is captured into a graph of the
+// caller's: replays run it at sweeps that only the device clock knows (they
+// then come after the clock's cursor, which k_advance keeps).  All 32 lanes call.
+constexpr uint32_t kScaReplayed = 0xFFFFFFFFu;
+struct ScaTimes {
+  uint32_t first, n;
+};
+__device__ __forceinline__ ScaTimes sca_times(const DomainLaunch& a, const ScaTileLaunch& t, uint64_t s0) {
+  const uint32_t next = a.clock->next_time;
+  if (t.rec_offset != kScaReplayed) return {next + t.rec_offset, t.n_rec};
+  const uint32_t lane = threadIdx.x & 31u;
+  // times are ascending: how many from `from` on are at most `last`, no more than `most`
+  const auto count = [&](uint32_t from, uint64_t last, uint32_t most) {
+    uint32_t n = 0;
+    for (uint32_t c = 32; c == 32u && n < most; n += c)
+      c = __popc(__ballot_sync(0xffffffffu, from + n + lane < a.n_times && a.times[from + n + lane] <= last));
+    return min(n, most);
+  };
+  const uint32_t first = next + count(next, s0, a.n_times);
+  return {first, count(first, s0 + t.n, t.n_rec)};
+}
 
 // The tile's hops since the launch began.
 __device__ __forceinline__ void tile_hops(const ScaCounts& cnt, ScaPart* part) {
@@ -235,7 +259,8 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
   ScaCounts cnt;
   const size_t part_pitch = static_cast<size_t>(a.geo.S) * t.tiles * NOCC;  // entries of one record
   ScaPart* part = t.parts + (static_cast<size_t>(sample) * t.tiles + tile) * NOCC;
-  const uint64_t* next_time = a.times + a.clock->next_time + t.rec_offset;
+  const ScaTimes rec_times = sca_times(a, t, s0);
+  const uint64_t* next_time = a.times + rec_times.first;
   uint32_t filled = 0, base = 0, recs = 0;
   for (uint32_t done = 0; done < t.n;) {
     if (done == filled) {
@@ -246,7 +271,7 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
       __syncwarp();
     }
     uint32_t stop = filled;
-    if (recs < t.n_rec) stop = static_cast<uint32_t>(min(static_cast<uint64_t>(stop), next_time[recs] - s0));
+    if (recs < rec_times.n) stop = static_cast<uint32_t>(min(static_cast<uint64_t>(stop), next_time[recs] - s0));
 #pragma unroll 1
     for (; done < stop; ++done) {
       const uint32_t it = done - base;
@@ -307,13 +332,12 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
                        : sca_turn_pool<1>(U[0][0], U[NOCC - 1][0], Q[0], *turn, gu[0], counted[0], a0, b2,
                                           hd[kmax + 1], a);
     }
-    if (recs < t.n_rec && next_time[recs] == s0 + done) {
-      tile_record<NOCC, UPT>(U, gu, counted, a, sample, s0 + done, part, COUNT, cnt);
-      part += part_pitch;
+    if (recs < rec_times.n && next_time[recs] == s0 + done) {
+      tile_record<NOCC, UPT>(U, gu, counted, a, sample, s0 + done, part + recs * part_pitch, COUNT, cnt);
       ++recs;
     }
   }
-  if (COUNT && t.n_rec) tile_hops(cnt, part);
+  if (COUNT && t.n_rec) tile_hops(cnt, part + t.n_rec * part_pitch);
 
 #pragma unroll
   for (uint32_t j = 0; j < UPT; ++j) {
@@ -350,7 +374,9 @@ __global__ void __launch_bounds__(128) k_sca_records(const DomainLaunch a, const
   const uint32_t S = a.geo.S, planes = a.geo.planes, n_units = a.geo.W / 8u;
   if (item >= static_cast<uint64_t>(t.n_rec) * S) return;  // whole warps
   const uint32_t r = static_cast<uint32_t>(item / S), sample = static_cast<uint32_t>(item - static_cast<uint64_t>(r) * S);
-  const size_t slot = static_cast<size_t>(a.clock->next_time) + t.rec_offset + r;
+  const ScaTimes times = sca_times(a, t, a.clock->sweep + t.offset);
+  if (r >= times.n) return;  // whole warps
+  const size_t slot = static_cast<size_t>(times.first) + r;
   const ScaPart* mine = t.parts + (static_cast<size_t>(r) * S + sample) * t.tiles * planes;
   const ScaPart* after = t.parts + (static_cast<size_t>(t.n_rec) * S + sample) * t.tiles * planes;
   long long hops[4] = {0, 0, 0, 0};
@@ -535,10 +561,11 @@ cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, const ScaRu
     t.tiles = tiles.tiles;
     t.units = tiles.units;
     t.n = std::min({kScaTileSweeps, run.max_sweeps, a.n_sweeps - done});
+    if (run.replayed && run.max_records) t.n = std::min(t.n, run.max_records);  // room for a record a sweep
     t.offset = done;
-    t.rec_offset = rec;
-    t.n_rec = 0;
-    while (rec + t.n_rec < run.n_times && run.times[rec + t.n_rec] - run.sweep <= done + t.n) {
+    t.rec_offset = run.replayed ? kScaReplayed : rec;
+    t.n_rec = run.replayed ? std::min(t.n, run.max_records) : 0u;
+    while (!run.replayed && rec + t.n_rec < run.n_times && run.times[rec + t.n_rec] - run.sweep <= done + t.n) {
       if (t.n_rec == run.max_records) {  // the launch ends before the first record it has no room for
         t.n = static_cast<uint32_t>(run.times[rec + t.n_rec - 1] - run.sweep) - done;
         break;
