@@ -681,7 +681,7 @@ def other_workloads(tune: bool = True, peak_ops: float | None = None, rng_bitop:
                               else "k_sca_tile"
                               if kw.get("schedule") == A.ASEP_SCHED_SCA
                               else "k_stream" if info["cluster"] == 32
-                              else "k_cluster" if info["cluster"] > 1 else "k_domain"),
+                              else "k_cluster" if A.asep_launch_cluster(ctx) > 1 else "k_domain"),
                    "samples_per_group": info["samples_per_group"]}
             if tuned:
                 row["plan"] = tuned

@@ -186,10 +186,12 @@ typedef struct asep_info {
   uint64_t attempts_per_sweep; /* L * planes per sample */
   uint64_t device_bytes;  /* device memory held by the context */
   uint64_t kernel_launches; /* kernels the context has enqueued so far */
+  /* The launch plan.  Launches of few samples under an automatic plan with cluster = 1 may be spread over
+     clusters all the same: asep_launch_cluster. */
   uint32_t cluster;       /* CTAs per sample: 1 = one CTA holds whole samples, 2..16 = a thread-block
                              cluster, 32 = streamed from global memory */
   uint32_t samples_per_group; /* samples per CTA (resident) or 1 (cluster) */
-  uint32_t groups;        /* CTAs (resident) or clusters per sweep launch */
+  uint32_t groups;        /* CTAs (resident) or clusters per sweep launch; SCA: tiles, a warp each */
   uint32_t threads;       /* threads per CTA */
   uint32_t smem_bytes;    /* dynamic shared memory per CTA of the sweep kernel */
   uint32_t tile_columns;  /* streamed domain tier: columns (threads) per tile; 0 otherwise */
@@ -294,6 +296,12 @@ int asep_height_offset(asep_ctx* ctx, int64_t* out, size_t n);
 /* Sizes, progress, device memory, launch count and launch plan of the
  * context (no synchronisation; n_recorded and sweep count enqueued work). */
 int asep_get_info(const asep_ctx* ctx, asep_info* info);
+
+/* CTAs per sample of the context's launches: asep_info.cluster, except that an
+ * automatic plan of whole samples in one CTA spreads few samples of at least
+ * 256 columns over clusters (asep_set_plan), which asep_info, whose launch
+ * plan is the one that bounds batches, does not show.  0 for NULL. */
+uint32_t asep_launch_cluster(const asep_ctx* ctx);
 
 /* Choose the launch plan of a context (the autotuner's knob; results never
  * depend on it).  Serial schedule: cluster 0 = automatic, 1 = one CTA per

@@ -97,7 +97,7 @@ EXPORTED = ("asep_create", "asep_plan", "asep_sweep", "asep_width", "asep_state"
             "asep_poisson_table", "asep_philox_bench", "asep_attempt_bench", "asep_version", "asep_batch_create", "asep_batch_sweep",
             "asep_batch_graph", "asep_batch_set_launch", "asep_batch_destroy", "asep_batch_last_error",
             "asep_batch_sweep_static", "asep_set_plan", "asep_set_launch_sweeps", "asep_set_balance", "asep_currents", "asep_profile", "asep_autocorr",
-            "asep_height_offset", "asep_inject_fault")
+            "asep_height_offset", "asep_inject_fault", "asep_launch_cluster")
 
 
 class AsepError(RuntimeError):
@@ -130,6 +130,8 @@ def lib():
             L.asep_counters.argtypes = [vp, P(ctypes.c_uint64), ctypes.c_size_t]
             L.asep_disorder.argtypes = [vp, P(ctypes.c_uint32), ctypes.c_size_t]
             L.asep_get_info.argtypes = [vp, P(asep_info)]
+            L.asep_launch_cluster.argtypes = [vp]
+            L.asep_launch_cluster.restype = ctypes.c_uint32
             L.asep_plan.argtypes = [P(asep_params), P(asep_info)]
             L.asep_sync.argtypes = [vp]
             L.asep_inject_fault.argtypes = [vp, ctypes.c_uint32]
@@ -340,6 +342,11 @@ def asep_get_info(ctx) -> dict:
     info = asep_info()
     _check(lib().asep_get_info(_h(ctx), ctypes.byref(info)), _h(ctx))
     return {f: getattr(info, f) for f, _ in asep_info._fields_}
+
+
+def asep_launch_cluster(ctx) -> int:
+    """CTAs per sample of the context's launches (an automatic one-CTA plan may spread few samples over clusters)."""
+    return int(lib().asep_launch_cluster(_h(ctx)))
 
 
 def asep_inject_fault(ctx, fault: int) -> None:

@@ -34,6 +34,9 @@ from . import asep as A
 
 @dataclass
 class Choice:
+    """`cluster` and `samples_per_group` (streamed plans: the tile width) as
+    ``asep_set_plan`` takes them; 0, 0 where the automatic plan spreads its
+    launches over clusters, which only the automatic plan does."""
     cluster: int
     samples_per_group: int
     ms_per_sweep: float
@@ -136,12 +139,16 @@ def autotune(ctx, probe_sweeps: int = 32, seed: int = 12345, launch_sweeps: bool
                 ref_words = words
             elif not np.array_equal(words, ref_words):
                 raise RuntimeError(f"plan cluster={cluster} spc={spc} balance={chunk} changed the result")
+            launched = A.asep_launch_cluster(ctx)
             second = info["tile_columns"] if info["cluster"] == 32 else info["samples_per_group"]
-            table.append({"knob": "plan", "cluster": info["cluster"], "samples_per_group": info["samples_per_group"],
-                          "tile_columns": info["tile_columns"], "balance_chunk_sweeps": chunk or "off",
-                          "ms_per_sweep": ms, "probe_sweeps": n, "requested": [cluster, spc]})
+            table.append({"knob": "plan", "cluster": info["cluster"], "launch_cluster": launched,
+                          "samples_per_group": info["samples_per_group"], "tile_columns": info["tile_columns"],
+                          "balance_chunk_sweeps": chunk or "off", "ms_per_sweep": ms, "probe_sweeps": n,
+                          "requested": [cluster, spc]})
             if best is None or ms < best_ms:
-                best, best_ms = Choice(info["cluster"], second, ms, 0, chunk), ms
+                automatic = launched != info["cluster"]  # spread: the plan that info names runs another kernel
+                best = Choice(0 if automatic else info["cluster"], 0 if automatic else second, ms, 0, chunk)
+                best_ms = ms
         A.asep_set_balance(ctx, 0)
     A.asep_set_plan(ctx, best.cluster, best.samples_per_group if best.cluster in (1, 32) else 0)
     A.asep_set_balance(ctx, best.balance)

@@ -1716,6 +1716,11 @@ int asep_get_info(const asep_ctx* ctx, asep_info* info) {
   return ASEP_OK;
 }
 
+uint32_t asep_launch_cluster(const asep_ctx* ctx) {
+  if (!ctx) return 0;
+  return ctx->spread.cluster && !ctx->balance ? ctx->spread.cluster : ctx->cluster;
+}
+
 int asep_destroy(asep_ctx* ctx) {
   if (!ctx) return ASEP_OK;
   release(ctx);

@@ -47,3 +47,35 @@ def test_plan_candidates_include_streamed_tile_widths(monkeypatch):
     assert not [x for x in autotune.candidates(None, sms=152) if x[0] == 32]
     monkeypatch.setattr(A, "asep_get_info", fake(65 * 64, 32, 4, 1))  # 130 words per plane: bulk copies need 4k
     assert not [x for x in autotune.candidates(None, sms=152) if x[0] == 32]
+
+
+def test_the_plan_applied_is_the_one_that_was_timed(monkeypatch):
+    """Few samples of 512 columns: the automatic plan reports one CTA and
+    launches clusters of four.  When it is the fastest it is applied as the
+    automatic plan, and stored so; (1, 1) would launch whole samples."""
+    calls, now = [], {"plan": (0, 0)}
+
+    def set_plan(ctx, cluster, spc):
+        now["plan"] = (cluster, spc)
+        calls.append((cluster, spc))
+
+    def info(ctx):
+        cluster, spc = now["plan"]
+        return {"L": 1 << 18, "D": 256, "S": 1, "cluster": cluster or 1, "samples_per_group": spc or 1, "groups": 1,
+                "tile_columns": spc if cluster == 32 else 0}
+
+    def probe(ctx, n, seed):
+        return {(0, 0): 0.030, (4, 0): 0.031}.get(now["plan"], 0.054), [0]
+
+    monkeypatch.setattr(A, "asep_set_plan", set_plan)
+    monkeypatch.setattr(A, "asep_get_info", info)
+    monkeypatch.setattr(A, "asep_launch_cluster", lambda ctx: 4 if now["plan"] == (0, 0) else max(1, now["plan"][0]),
+                        raising=False)
+    monkeypatch.setattr(A, "asep_set_balance", lambda ctx, chunk: None)
+    monkeypatch.setattr(A, "asep_set_launch_sweeps", lambda ctx, cap: None)
+    monkeypatch.setattr(autotune, "_probe", probe)
+    monkeypatch.setattr(autotune, "_sm_count", lambda: 152)
+    choice, table = autotune.autotune(None)
+    assert calls[-1] == (0, 0) and (choice.cluster, choice.samples_per_group) == (0, 0)
+    assert choice.ms_per_sweep == 0.030
+    assert all(r["ms_per_sweep"] == 0.030 for r in table if r["knob"] == "launch_sweeps")

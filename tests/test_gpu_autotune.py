@@ -118,3 +118,17 @@ def test_autotune_times_the_launch_sweeps_and_batch_mode():
     mode, rows = autotune.tune_batch_mode(make, [4] * len(shapes), steps=5)
     assert mode in ("eager", "graph") and [r["mode"] for r in rows] == ["eager", "graph"]
     assert all(r["ms_per_step"] > 0 for r in rows)
+
+
+@pytest.mark.parametrize("G", [128, 512])
+def test_the_plan_applied_launches_what_was_timed(G):
+    """One ring of 512 columns, whose automatic plan launches clusters, and one of 128."""
+    with A.asep_create(A.make_params(L=512 * G, domain_sites=256, p_thr=th(0.7)), sample_times=[]) as ctx:
+        assert (A.asep_launch_cluster(ctx) > 1) == (G == 512) and A.asep_get_info(ctx)["cluster"] == 1
+        choice, table = autotune.autotune(ctx, probe_sweeps=16)
+        best = min((r for r in table if r["knob"] == "plan"), key=lambda r: r["ms_per_sweep"])
+        assert A.asep_launch_cluster(ctx) == best["launch_cluster"]
+        A.asep_set_plan(ctx, 1, 0)
+        assert A.asep_launch_cluster(ctx) == 1
+        A.asep_set_plan(ctx, choice.cluster, choice.samples_per_group if choice.cluster in (1, 32) else 0)
+        assert A.asep_launch_cluster(ctx) == best["launch_cluster"]
