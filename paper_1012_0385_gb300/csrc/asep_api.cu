@@ -276,9 +276,9 @@ int plan_sca(asep_ctx* ctx, uint32_t force) {
 // Bytes of the tiles' edge buffer.
 size_t sca_halo_bytes(const asep_ctx* ctx) { return sca_halo_words(ctx->sca, ctx->S, ctx->planes) * 4u; }
 
-// Bytes of the tiles' parts of a launch's records (none without sample times).
+// Bytes of the tiles' parts of a launch's records (none without sample times or for rings of one tile).
 size_t sca_parts_bytes(const asep_ctx* ctx) {
-  if (!ctx->sca_records) return 0;
+  if (!ctx->sca_records || ctx->sca.tiles == 1) return 0;
   return (ctx->sca_records + static_cast<size_t>(1)) * ctx->S * ctx->sca.tiles * ctx->planes * sizeof(ScaPart);
 }
 

@@ -255,7 +255,7 @@ struct ScaTiles {
   uint32_t tiles, units, upt;  // tiles per ring, units (of 8 words) per tile, units per thread
 };
 ScaTiles sca_tiles(uint32_t model, uint32_t dis, uint32_t p_thr, uint32_t q_thr, uint32_t W, uint32_t S);
-// Words of the buffer of the tiles' edge units, two halves.
+// Words of the buffer of the tiles' edge units, two halves (none for rings of one tile).
 size_t sca_halo_words(const ScaTiles& t, uint32_t S, uint32_t planes);
 // A tile's part of a record: height change and sums of its heights relative
 // to its entry height, autocorrelation overlap, and (plane 0) its hops since
@@ -266,7 +266,8 @@ struct ScaPart {
   uint64_t s2;
   uint32_t hops[4];
 };
-// Records one launch holds at most: as many as fall into it, within 64 MB.
+// Records one launch holds at most: as many as fall into it, within 64 MB of
+// parts (rings of one tile need none).
 uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t tiles, uint32_t planes);
 // One call's buffers and schedule (host).
 struct ScaRun {

@@ -58,9 +58,9 @@ struct ScaTileLaunch {
   uint32_t n, offset;     // sweeps of this launch, and before it since the context clock
   uint32_t n_rec, rec_offset;  // sample times inside this launch, and before it since the clock's cursor
                                // (kScaReplayed: the device finds them, at most n_rec)
-  const uint32_t* halo_in;   // [S][tiles][first, last unit][planes][8]
+  const uint32_t* halo_in;   // [S][tiles][first, last unit][planes][8] (one tile a ring: unused)
   uint32_t* halo_out;
-  ScaPart* parts;         // [n_rec + 1][S][tiles][planes] (the last entry: the launch's hops)
+  ScaPart* parts;         // [n_rec + 1][S][tiles][planes] (the last entry: the launch's hops; one tile: unused)
 };
 
 // ---------------------------------------------------------------------------
@@ -92,6 +92,11 @@ struct ScaTileLaunch {
 // between launches -- the launch, k_heights, the clock, the next launch --
 // took some 25 us; 256 rings of 2^17 with 88 log-spaced records in 2048
 // sweeps spent 2.2 of 5.6 ms there.)
+//
+// A ring of one tile is its own neighbour: its halos come from its own units of
+// the lattice, and a record of it is whole.  It needs neither buffer, which are
+// 128 B of halo a tile and plane and 40 B a record, tile and plane beside 32 B
+// of lattice a unit.
 
 // Sample times of a launch from sweep s0 on: index of the first, and how many.
 // The host knows both, except of a launch that is captured into a graph of the
@@ -125,11 +130,12 @@ __device__ __forceinline__ void tile_hops(const ScaCounts& cnt, ScaPart* part) {
   }
 }
 
-// One record of one tile: the other observables, and its part of the height sums.
+// One record of one tile: the other observables, and its part of the height
+// sums, or (one tile a ring) the record itself, in slot `slot`.
 template <uint32_t NOCC, uint32_t UPT>
 __device__ void tile_record(const ScaUnit (&U)[NOCC][UPT], const uint32_t (&gu)[UPT], const uint32_t (&counted)[UPT],
-                            const DomainLaunch& a, uint32_t sample, uint64_t time, ScaPart* part, bool count,
-                            const ScaCounts& cnt) {
+                            const DomainLaunch& a, uint32_t sample, uint64_t time, size_t slot, bool whole,
+                            ScaPart* part, bool count, const ScaCounts& cnt) {
   const uint32_t lane = threadIdx.x & 31u;
   const Extras& ex = a.ex;
 #pragma unroll
@@ -178,14 +184,31 @@ __device__ void tile_record(const ScaUnit (&U)[NOCC][UPT], const uint32_t (&gu)[
       s2 += __shfl_xor_sync(0xffffffffu, s2, d);
       ov += __shfl_xor_sync(0xffffffffu, ov, d);
     }
-    if (lane == 31u) {
+    if (whole) {
+      if (lane == 31u) {
+        const size_t e = (slot * a.geo.S + sample) * NOCC + p;
+        a.tab_sh[e] = s1;
+        a.tab_sh2[2 * e] = s2;
+        a.tab_sh2[2 * e + 1] = 0;
+        if (ex.snap) ex.tab_ac[e] = ov;
+      }
+    } else if (lane == 31u) {
       part[p].tot = incl;
       part[p].ov = ov;
       part[p].s1 = s1;
       part[p].s2 = s2;
     }
   }
-  if (count) tile_hops(cnt, part);
+  if (whole) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const uint32_t v = __reduce_add_sync(0xffffffffu, cnt.c[k]);  // since the launch began
+      if (lane == 31u)
+        ex.tab_cnt[(slot * a.geo.S + sample) * 4 + k] = static_cast<int64_t>(a.counters[4ull * sample + k] + v);
+    }
+  } else if (count) {
+    tile_hops(cnt, part);
+  }
 }
 
 template <uint32_t MODEL, bool DIS, bool COUNT, uint32_t FAST, bool PQ, uint32_t UPT>
@@ -224,7 +247,7 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
     counted[j] = own ? ~0u : 0u;
     const uint32_t* src = state + 8u * g;
     size_t pitch = W;
-    if (used && !own) {  // left halo: the previous tile's last unit; right halo: the next tile's first
+    if (used && !own && t.tiles > 1u) {  // left halo: the previous tile's last unit; right halo: the next tile's first
       const uint32_t nb = i == 0u ? (tile == 0u ? t.tiles : tile) - 1u : (tile + 1u == t.tiles ? 0u : tile + 1u);
       src = t.halo_in + (edge0 + 2u * nb + (i == 0u ? 1u : 0u)) * (NOCC * 8u);
       pitch = 8;
@@ -333,11 +356,12 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
                                           hd[kmax + 1], a);
     }
     if (recs < rec_times.n && next_time[recs] == s0 + done) {
-      tile_record<NOCC, UPT>(U, gu, counted, a, sample, s0 + done, part + recs * part_pitch, COUNT, cnt);
+      tile_record<NOCC, UPT>(U, gu, counted, a, sample, s0 + done, rec_times.first + recs, t.tiles == 1u,
+                             part + recs * part_pitch, COUNT, cnt);
       ++recs;
     }
   }
-  if (COUNT && t.n_rec) tile_hops(cnt, part + t.n_rec * part_pitch);
+  if (COUNT && t.n_rec && t.tiles > 1u) tile_hops(cnt, part + t.n_rec * part_pitch);
 
 #pragma unroll
   for (uint32_t j = 0; j < UPT; ++j) {
@@ -348,6 +372,7 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
       uint32_t x[8];
       to_words(U[p][j], x);
       store8(state + p * W + 8u * gu[j], x);
+      if (t.tiles == 1u) continue;
       if (i == 1u) store8(t.halo_out + ((edge0 + 2u * tile) * NOCC + p) * 8u, x);
       if (i == n_own) store8(t.halo_out + ((edge0 + 2u * tile + 1u) * NOCC + p) * 8u, x);
     }
@@ -529,7 +554,7 @@ ScaTiles sca_tiles(uint32_t model, uint32_t dis, uint32_t p_thr, uint32_t q_thr,
 }
 
 size_t sca_halo_words(const ScaTiles& t, uint32_t S, uint32_t planes) {
-  return static_cast<size_t>(2u) * S * t.tiles * 2u * planes * 8u;
+  return t.tiles == 1u ? 0u : static_cast<size_t>(2u) * S * t.tiles * 2u * planes * 8u;
 }
 
 uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t tiles, uint32_t planes) {
@@ -538,6 +563,7 @@ uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t t
     while (times[j] - times[i] >= kScaTileSweeps) ++i;
     most = std::max(most, static_cast<uint32_t>(j - i + 1));
   }
+  if (tiles == 1u) return most;  // written by the tiles themselves
   // no more than 64 MB or a record's worth
   const uint64_t one = static_cast<uint64_t>(S) * tiles * planes * sizeof(ScaPart);
   return static_cast<uint32_t>(std::min<uint64_t>(most, std::max<uint64_t>(1u, (64ull << 20) / one)));
@@ -547,8 +573,8 @@ cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, const ScaRu
                        uint32_t* launches) {
   const size_t half = sca_halo_words(tiles, a.geo.S, a.geo.planes) / 2u;
   uint32_t parity = 0, rec = 0;
-  {
-    (void)cudaGetLastError();
+  (void)cudaGetLastError();
+  if (tiles.tiles > 1u) {
     const size_t n16 = half / 4u;
     const uint32_t blocks = static_cast<uint32_t>(std::min<size_t>((n16 + 255u) / 256u, 152u * 16u));
     k_sca_halo<<<blocks, 256, 0, st>>>(a.state, run.halo, a.geo.S, a.geo.planes, a.geo.W, tiles.tiles, tiles.units);
@@ -578,7 +604,7 @@ cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, const ScaRu
     cudaError_t e = launch_tiles(a, t, tiles.upt, st);
     if (e != cudaSuccess) return e;
     ++*launches;
-    if (t.n_rec) {
+    if (t.n_rec && tiles.tiles > 1u) {
       const uint64_t items = static_cast<uint64_t>(t.n_rec) * a.geo.S;
       k_sca_records<<<static_cast<uint32_t>((items + 3u) / 4u), 128, 0, st>>>(a, t);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
