@@ -78,6 +78,7 @@ struct asep_ctx {
   uint32_t balance = 0;            // balanced launches: sweeps per chunk (0 = off)
   ScaTiles sca{};                  // SCA: tiles of a ring
   uint32_t* d_halo = nullptr;      // SCA: the tiles' edge units, two halves
+  uint32_t halo_half = kScaNoHalo; // ... the one that holds those of d_state (kScaNoHalo: the lattice was replaced)
   uint32_t sca_records = 0;        // SCA: records a launch holds at most
   ScaPart* d_sca_parts = nullptr;  // SCA: the tiles' parts of a launch's records
   bool replayed = false;           // asep_sweep was captured into a caller's graph: the device clock alone is right
@@ -962,7 +963,7 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
   uint64_t done = 0;
   while (done < n_mcs) {
     uint64_t n = n_mcs - done;
-    uint32_t sweep_launches = 0;  // SCA: counted by the launch
+    uint32_t sweep_launches = 0;  // SCA: counted by the launch, with the clock's
     const uint32_t cap = sweeps_cap(ctx);
     if (ctx->p.schedule == ASEP_SCHED_SCA) n = std::min<uint64_t>(n, 1u << 20);  // split into launches there
     else if (n > cap) n = cap;
@@ -984,6 +985,7 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
       ScaRun run;
       run.replayed = capturing || (ctx->replayed && ctx->next_time < ctx->times.size());
       run.halo = ctx->d_halo;
+      run.half = ctx->replayed ? kScaNoHalo : ctx->halo_half;  // replays move the lattice on without the host
       run.parts = ctx->d_sca_parts;
       run.max_records = ctx->sca_records;
       run.max_sweeps = cap;
@@ -991,6 +993,7 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
       run.times = ctx->times.data() + ctx->next_time;
       run.n_times = ctx->times.size() - ctx->next_time;
       e = launch_sca(domain_desc(ctx, static_cast<uint32_t>(n)), ctx->sca, run, ctx->stream, &sweep_launches);
+      ctx->halo_half = run.half;
     } else if (ctx->p.schedule == ASEP_SCHED_DOMAIN && ctx->balance && ctx->cluster == 1 && n > ctx->balance) {
       BalanceLaunch b;
       b.chunk = ctx->balance;
@@ -1024,15 +1027,16 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
       e = launch_serial_plan(a, ctx->p.model, ctx->p.dis_kind, ctx->cluster, ctx->stream);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "sweep kernel launch");
-    if ((e = launch_advance(ctx->d_clock, ctx->d_times, static_cast<uint32_t>(ctx->times.size()),
-                            static_cast<uint32_t>(n), ctx->stream)) != cudaSuccess)
-      return cuda_fail(ctx, e, "clock advance");
-    // the sweep kernels (streamed domain tier: one per phase, plus the lane
-    // changes with turning sites) and the clock
-    if (ctx->p.schedule != ASEP_SCHED_SCA)
-      sweep_launches = ctx->cluster != kStreamTier ? 1u
-                       : (ctx->p.dis_kind == ASEP_DIS_TURNING || ctx->p.dis_kind == ASEP_DIS_CROSSING) ? 3u : 2u;
-    ctx->launches += sweep_launches + 1;
+    if (ctx->p.schedule != ASEP_SCHED_SCA) {
+      if ((e = launch_advance(ctx->d_clock, ctx->d_times, static_cast<uint32_t>(ctx->times.size()),
+                              static_cast<uint32_t>(n), ctx->stream)) != cudaSuccess)
+        return cuda_fail(ctx, e, "clock advance");
+      // the sweep kernels (streamed domain tier: one per phase, plus the lane
+      // changes with turning sites) and the clock
+      sweep_launches = ctx->cluster != kStreamTier ? 2u
+                       : (ctx->p.dis_kind == ASEP_DIS_TURNING || ctx->p.dis_kind == ASEP_DIS_CROSSING) ? 4u : 3u;
+    }
+    ctx->launches += sweep_launches;
     advance_host(ctx, n);
     done += n;
   }
@@ -1058,6 +1062,7 @@ int asep_reset(asep_ctx* ctx, uint64_t seed, uint64_t init_seed) {
   InitLaunch il;
   il.geo = geometry(ctx);
   il.state = ctx->d_state;
+  ctx->halo_half = kScaNoHalo;
   il.init_kind = ctx->p.init_kind;
   il.init_seed = init_seed;
   if ((e = launch_init(il, ctx->stream)) != cudaSuccess) return cuda_fail(ctx, e, "init kernel");
@@ -1155,6 +1160,7 @@ int asep_load_state(asep_ctx* ctx, const uint32_t* words, size_t n_words, uint64
   if (sweep >= (1ull << 40)) return fail(ctx, ASEP_ERR_INVALID, "sweep index >= 2^40");
   int rc = clear_timeout(ctx);  // the loaded state replaces results a timed-out sweep invalidated
   if (rc != ASEP_OK) return rc;
+  ctx->halo_half = kScaNoHalo;
   const cudaError_t e = cudaMemcpy(ctx->d_state, words, need * 4, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "load state");
   if ((rc = record_reference(ctx)) != ASEP_OK) return rc;

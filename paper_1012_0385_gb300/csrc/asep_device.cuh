@@ -113,6 +113,15 @@ __device__ __forceinline__ uint32_t pick(const uint4 x, uint32_t i) {
 // A draw r accepts a move of threshold t (0, a multiple of 4096 or "always").
 __device__ __forceinline__ bool accept(uint32_t r, uint32_t t) { return (r & kAcceptMask) < t; }
 
+// Moves the clock n sweeps on (one thread).
+__device__ __forceinline__ void advance_clock(Clock* c, const uint64_t* times, uint32_t n_times, uint32_t n) {
+  const unsigned long long sweep = c->sweep + n;
+  uint32_t next = c->next_time;
+  while (next < n_times && times[next] <= sweep) ++next;
+  c->sweep = sweep;
+  c->next_time = next;
+}
+
 // ---------------------------------------------------------------------------
 // Heights of a word
 // ---------------------------------------------------------------------------

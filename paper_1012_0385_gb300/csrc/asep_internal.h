@@ -59,7 +59,7 @@ inline int32_t hop_bound(uint32_t t) {
 struct Clock {
   unsigned long long sweep;
   uint32_t next_time;
-  uint32_t pad;
+  uint32_t done;  // blocks through with a launch whose last one moves the clock; zero between launches
 };
 
 struct Geometry {
@@ -269,19 +269,22 @@ struct ScaPart {
 // Records one launch holds at most: as many as fall into it, within 64 MB of
 // parts (rings of one tile need none).
 uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t tiles, uint32_t planes);
+constexpr uint32_t kScaNoHalo = 2;
 // One call's buffers and schedule (host).
 struct ScaRun {
   uint32_t* halo;          // sca_halo_words words
   ScaPart* parts;          // [max_records + 1][S][tiles][planes]
+  uint32_t half;           // the half of the buffer that holds the lattice's edge units, before and after the call
+                           // (kScaNoHalo: neither)
   uint32_t max_records, max_sweeps;  // per launch
   uint64_t sweep;          // sweep count at the start of the call
   const uint64_t* times;   // the sample times not yet recorded
   size_t n_times;
   bool replayed;           // the launches may run at other sweeps than the host's (captured into a caller's graph)
 };
-// a.n_sweeps sweeps in launches of at most 128, with the records inside them;
-// *launches is advanced.
-cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, const ScaRun& run, cudaStream_t st,
+// a.n_sweeps sweeps in launches of at most 128, with the records inside them,
+// and the clock moved past them; *launches is advanced.
+cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, ScaRun& run, cudaStream_t st,
                        uint32_t* launches);
 // The bound by which the one-CTA plan code is offered: lattice, classes and
 // carries within 200 KB.

@@ -226,14 +226,6 @@ __global__ void __launch_bounds__(1024, 1) k_domain(const DomainLaunch a) {
   run_group<MODEL, DIS, COUNT, CP>(a, blockIdx.x, smem_raw, a.clock->sweep, a.clock->next_time, a.n_sweeps);
 }
 
-__device__ __forceinline__ void advance_clock(Clock* c, const uint64_t* times, uint32_t n_times, uint32_t n) {
-  const unsigned long long sweep = c->sweep + n;
-  uint32_t next = c->next_time;
-  while (next < n_times && times[next] <= sweep) ++next;
-  c->sweep = sweep;
-  c->next_time = next;
-}
-
 __global__ void k_advance(Clock* clock, const uint64_t* times, uint32_t n_times, uint32_t n) {
   if (blockIdx.x == 0 && threadIdx.x == 0) advance_clock(clock, times, n_times, n);
 }
@@ -242,6 +234,7 @@ __global__ void k_set_clock(Clock* clock, unsigned long long sweep, uint32_t nex
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     clock->sweep = sweep;
     clock->next_time = next_time;
+    clock->done = 0u;
   }
 }
 

@@ -77,7 +77,8 @@ struct ScaTileLaunch {
 // sweep.  One tile a CTA, so that tiles spread over the SMs evenly.
 // In place: a tile reads and writes only its own units of the lattice; its
 // neighbours' edge units come from a buffer that the previous launch (or
-// k_sca_halo, at the start of a call) filled, and go to the other half of it.
+// k_sca_halo, once the lattice was replaced) filled, and go to the other half of
+// it.
 // Bound by the integer ALU pipe (logic of Philox and of the update: 69 % busy,
 // 173 of 268 instructions a unit and sweep at two planes).  Measured against
 // one CTA per ring with two barriers a sweep, and against one launch per phase
@@ -393,7 +394,10 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
 // with their entry heights H_j added back exactly (sum (H + h') = sum h' + H n,
 // sum (H + h')^2 = sum h'^2 + 2 H sum h' + H^2 n), and the hop counters at the
 // record: those after the launch, less the launch's hops, plus its hops so far.
-__global__ void __launch_bounds__(128) k_sca_records(const DomainLaunch a, const ScaTileLaunch t) {
+// advance: sweeps that the last block to end moves the clock by (0 = none): every
+// block has read it by then.  (A launch for the clock alone is 2 us of the some
+// 17 of a call of one sweep of a small context.)
+__device__ __forceinline__ void sca_records(const DomainLaunch& a, const ScaTileLaunch& t) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint64_t item = static_cast<uint64_t>(blockIdx.x) * 4u + (threadIdx.x >> 5);
   const uint32_t S = a.geo.S, planes = a.geo.planes, n_units = a.geo.W / 8u;
@@ -457,6 +461,15 @@ __global__ void __launch_bounds__(128) k_sca_records(const DomainLaunch a, const
       a.ex.tab_cnt[(slot * S + sample) * 4 + k] =
           static_cast<int64_t>(a.counters[4ull * sample + k]) + hops[k];
   }
+}
+
+__global__ void __launch_bounds__(128) k_sca_records(const DomainLaunch a, const ScaTileLaunch t, uint32_t advance) {
+  sca_records(a, t);
+  if (!advance) return;
+  __syncthreads();
+  __threadfence();
+  if (threadIdx.x == 0u && atomicInc(&a.clock->done, gridDim.x - 1u) == gridDim.x - 1u)
+    advance_clock(a.clock, a.times, a.n_times, advance);
 }
 
 // The first and last unit of every tile, from the lattice: one thread per 16 bytes.
@@ -569,12 +582,13 @@ uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t t
   return static_cast<uint32_t>(std::min<uint64_t>(most, std::max<uint64_t>(1u, (64ull << 20) / one)));
 }
 
-cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, const ScaRun& run, cudaStream_t st,
+cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, ScaRun& run, cudaStream_t st,
                        uint32_t* launches) {
   const size_t half = sca_halo_words(tiles, a.geo.S, a.geo.planes) / 2u;
-  uint32_t parity = 0, rec = 0;
+  uint32_t rec = 0;
+  bool advanced = false;
   (void)cudaGetLastError();
-  if (tiles.tiles > 1u) {
+  if (tiles.tiles > 1u && run.half == kScaNoHalo) {
     const size_t n16 = half / 4u;
     const uint32_t blocks = static_cast<uint32_t>(std::min<size_t>((n16 + 255u) / 256u, 152u * 16u));
     k_sca_halo<<<blocks, 256, 0, st>>>(a.state, run.halo, a.geo.S, a.geo.planes, a.geo.W, tiles.tiles, tiles.units);
@@ -582,6 +596,8 @@ cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, const ScaRu
     if (e != cudaSuccess) return e;
     ++*launches;
   }
+  uint32_t half_now = run.half == kScaNoHalo ? 0u : run.half;
+  run.half = kScaNoHalo;  // until all is launched
   for (uint32_t done = 0; done < a.n_sweeps;) {
     ScaTileLaunch t;
     t.tiles = tiles.tiles;
@@ -598,22 +614,29 @@ cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, const ScaRu
       }
       ++t.n_rec;
     }
-    t.halo_in = run.halo + parity * half;
-    t.halo_out = run.halo + (parity ^ 1u) * half;
+    t.halo_in = run.halo + half_now * half;
+    t.halo_out = run.halo + (half_now ^ 1u) * half;
     t.parts = run.parts;
     cudaError_t e = launch_tiles(a, t, tiles.upt, st);
     if (e != cudaSuccess) return e;
     ++*launches;
     if (t.n_rec && tiles.tiles > 1u) {
       const uint64_t items = static_cast<uint64_t>(t.n_rec) * a.geo.S;
-      k_sca_records<<<static_cast<uint32_t>((items + 3u) / 4u), 128, 0, st>>>(a, t);
+      advanced = done + t.n == a.n_sweeps;
+      k_sca_records<<<static_cast<uint32_t>((items + 3u) / 4u), 128, 0, st>>>(a, t, advanced ? a.n_sweeps : 0u);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
       ++*launches;
     }
-    parity ^= 1u;
+    half_now ^= 1u;
     rec += t.n_rec;
     done += t.n;
   }
+  if (!advanced) {
+    const cudaError_t e = launch_advance(a.clock, a.times, a.n_times, a.n_sweeps, st);
+    if (e != cudaSuccess) return e;
+    ++*launches;
+  }
+  run.half = half_now;
   return cudaSuccess;
 }
 
