@@ -80,6 +80,7 @@ struct asep_ctx {
   uint32_t* d_halo = nullptr;      // SCA: the tiles' edge units, two halves
   uint32_t halo_half = kScaNoHalo; // ... the one that holds those of d_state (kScaNoHalo: the lattice was replaced)
   uint32_t sca_records = 0;        // SCA: records a launch holds at most
+  uint32_t sca_any_sweeps = 1;     // SCA: sweeps a launch holds the records of wherever it begins
   ScaPart* d_sca_parts = nullptr;  // SCA: the tiles' parts of a launch's records
   bool replayed = false;           // asep_sweep was captured into a caller's graph: the device clock alone is right
   uint32_t* d_progress = nullptr;  // balanced launches: [S + 1] chunk flags and queue counter
@@ -267,7 +268,8 @@ int plan_sca(asep_ctx* ctx, uint32_t force) {
                 "takes %zu bytes)", smem);
   ctx->cluster = force != kStreamTier && fits ? 1u : kStreamTier;
   ctx->sca = sca_tiles(ctx->p.model, ctx->p.dis_kind, ctx->p.p_thr, ctx->p.q_thr, ctx->W, ctx->S);
-  ctx->sca_records = sca_max_records(ctx->times.data(), ctx->times.size(), ctx->S, ctx->sca.tiles, ctx->planes);
+  ctx->sca_records = sca_max_records(ctx->times.data(), ctx->times.size(), ctx->S, ctx->sca.tiles, ctx->planes,
+                                     &ctx->sca_any_sweeps);
   ctx->threads = 32;
   ctx->smem = 0;
   ctx->blocks = ctx->S * ctx->sca.tiles;
@@ -989,6 +991,7 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
       run.parts = ctx->d_sca_parts;
       run.max_records = ctx->sca_records;
       run.max_sweeps = cap;
+      run.any_sweeps = ctx->sca_any_sweeps;
       run.sweep = ctx->sweep;
       run.times = ctx->times.data() + ctx->next_time;
       run.n_times = ctx->times.size() - ctx->next_time;

@@ -267,8 +267,10 @@ struct ScaPart {
   uint32_t hops[4];
 };
 // Records one launch holds at most: as many as fall into it, within 64 MB of
-// parts (rings of one tile need none).
-uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t tiles, uint32_t planes);
+// parts (rings of one tile need none).  *any_sweeps: a launch of no more sweeps
+// has room for its records wherever it begins.
+uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t tiles, uint32_t planes,
+                         uint32_t* any_sweeps);
 constexpr uint32_t kScaNoHalo = 2;
 // One call's buffers and schedule (host).
 struct ScaRun {
@@ -277,6 +279,7 @@ struct ScaRun {
   uint32_t half;           // the half of the buffer that holds the lattice's edge units, before and after the call
                            // (kScaNoHalo: neither)
   uint32_t max_records, max_sweeps;  // per launch
+  uint32_t any_sweeps;     // per launch that may run at other sweeps than the host's
   uint64_t sweep;          // sweep count at the start of the call
   const uint64_t* times;   // the sample times not yet recorded
   size_t n_times;

@@ -570,7 +570,9 @@ size_t sca_halo_words(const ScaTiles& t, uint32_t S, uint32_t planes) {
   return t.tiles == 1u ? 0u : static_cast<size_t>(2u) * S * t.tiles * 2u * planes * 8u;
 }
 
-uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t tiles, uint32_t planes) {
+uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t tiles, uint32_t planes,
+                         uint32_t* any_sweeps) {
+  *any_sweeps = kScaTileSweeps;
   uint32_t most = 0;  // sample times in any kScaTileSweeps consecutive sweeps
   for (size_t i = 0, j = 0; j < n; ++j) {
     while (times[j] - times[i] >= kScaTileSweeps) ++i;
@@ -579,7 +581,10 @@ uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t t
   if (tiles == 1u) return most;  // written by the tiles themselves
   // no more than 64 MB or a record's worth
   const uint64_t one = static_cast<uint64_t>(S) * tiles * planes * sizeof(ScaPart);
-  return static_cast<uint32_t>(std::min<uint64_t>(most, std::max<uint64_t>(1u, (64ull << 20) / one)));
+  const uint64_t room = std::max<uint64_t>(1u, (64ull << 20) / one);
+  if (room >= most) return most;
+  *any_sweeps = static_cast<uint32_t>(room);  // at most a record a sweep
+  return static_cast<uint32_t>(room);
 }
 
 cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, ScaRun& run, cudaStream_t st,
@@ -603,7 +608,7 @@ cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, ScaRun& run
     t.tiles = tiles.tiles;
     t.units = tiles.units;
     t.n = std::min({kScaTileSweeps, run.max_sweeps, a.n_sweeps - done});
-    if (run.replayed && run.max_records) t.n = std::min(t.n, run.max_records);  // room for a record a sweep
+    if (run.replayed) t.n = std::min(t.n, run.any_sweeps);
     t.offset = done;
     t.rec_offset = run.replayed ? kScaReplayed : rec;
     t.n_rec = run.replayed ? std::min(t.n, run.max_records) : 0u;

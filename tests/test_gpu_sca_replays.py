@@ -67,3 +67,25 @@ def test_replays(kind, times, units):
         assert np.array_equal(words, A.asep_state(ctx)[0])
         for x, y in zip(got, outputs(ctx)):
             assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("times", ["late", "all", "dense"])
+def test_captured_launches_are_as_long_as_others(times):
+    """Two tiles a ring, 260 sweeps captured: three launches of the tiles, each
+    with one for the records, however few sample times there are; a record
+    buffer short of 128 records (6700 rings) cuts them to what it holds."""
+    import torch
+
+    for samples, most in [(2, 128), (6700, 125)]:
+        kw = dict(schedule=A.ASEP_SCHED_SCA, L=256 * 31, samples_per_real=samples, seed=1, **KINDS["ring"])
+        stream = torch.cuda.Stream()
+        every = list(range(1, 400)) if samples > 2 else TIMES[times]
+        with A.asep_create(A.make_params(**kw), sample_times=every, stream=stream.cuda_stream) as ctx:
+            A.asep_sweep(ctx, 1)
+            before = A.asep_get_info(ctx)["kernel_launches"]
+            graph = torch.cuda.CUDAGraph()
+            torch.cuda.synchronize()
+            with torch.cuda.graph(graph, stream=stream):
+                A.asep_sweep(ctx, 260)
+            launches = A.asep_get_info(ctx)["kernel_launches"] - before
+            assert launches <= 1 + 2 * -(-260 // most)
