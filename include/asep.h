@@ -218,7 +218,13 @@ int asep_plan(const asep_params* params, asep_info* info);
 /* Enqueue n_mcs sweeps (Monte Carlo steps, paper sec. 2.1: one sweep = L
  * attempts per lane and sample) of all S samples on the context stream,
  * recording heights after every sweep count listed in sample_times.
- * Asynchronous: returns once the work is enqueued. */
+ * Asynchronous: returns once the work is enqueued (the SCA puts a call of more
+ * than 256 launches, 32768 sweeps, on the stream as CUDA graphs, so that it
+ * fits the stream's queue; making them takes the host 0.5 to 6 ms).  A call may
+ * be captured into a CUDA graph of the caller's: replays continue from the
+ * device's sweep count, but what the host reports (asep_info, how many records
+ * the tables hold) counts calls, not replays, until asep_load_state or
+ * asep_reset sets both. */
 int asep_sweep(asep_ctx* ctx, uint64_t n_mcs);
 
 /* Copy the heights recorded so far.  Entry e = (time index, sample, plane),
@@ -329,7 +335,7 @@ int asep_set_plan(asep_ctx* ctx, uint32_t cluster, uint32_t samples_per_group);
 
 /* Cap the sweeps one kernel launch (or one batch step) runs for this
  * context: max_sweeps = 0 restores the automatic bound (the 32-bit per-lane
- * hop counters of the domain schedule, 2^20 otherwise).  Longer asep_sweep
+ * hop counters of the domain schedule, 128 of the SCA, 2^20 of the serial one).  Longer asep_sweep
  * and batch calls are split into launches of at most this many sweeps; the
  * streamed domain tier runs one sweep per step whatever the cap.  An autotuner knob:
  * results never depend on it (every sample's randomness is keyed by its

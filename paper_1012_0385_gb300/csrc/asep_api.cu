@@ -78,6 +78,7 @@ struct asep_ctx {
   uint32_t balance = 0;            // balanced launches: sweeps per chunk (0 = off)
   ScaTiles sca{};                  // SCA: tiles of a ring
   uint32_t* d_halo = nullptr;      // SCA: the tiles' edge units, two halves
+  cudaStream_t cap_stream = nullptr;  // SCA: long calls are captured here
   uint32_t halo_half = kScaNoHalo; // ... the one that holds those of d_state (kScaNoHalo: the lattice was replaced)
   uint32_t sca_records = 0;        // SCA: records a launch holds at most
   uint32_t sca_any_sweeps = 1;     // SCA: sweeps a launch holds the records of wherever it begins
@@ -207,6 +208,8 @@ void release(asep_ctx* ctx) {
     }
   }
   ctx->allocs.clear();
+  if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
+  ctx->cap_stream = nullptr;
 }
 
 int validate(const asep_params* p, asep_ctx* ctx) {
@@ -653,6 +656,135 @@ void advance_host(asep_ctx* ctx, uint64_t n) {
   while (ctx->next_time < ctx->times.size() && ctx->times[ctx->next_time] <= ctx->sweep) ++ctx->next_time;
 }
 
+// SCA: n sweeps from the host's clock on as launches on the context's stream.
+int sca_direct(asep_ctx* ctx, uint64_t n, bool capturing) {
+  while (n) {
+    const uint32_t step = static_cast<uint32_t>(std::min<uint64_t>(n, 1u << 20));
+    ScaRun run;
+    run.replayed = capturing || (ctx->replayed && ctx->next_time < ctx->times.size());
+    run.halo = ctx->d_halo;
+    run.half = ctx->replayed ? kScaNoHalo : ctx->halo_half;  // replays move the lattice on without the host
+    run.parts = ctx->d_sca_parts;
+    run.max_records = ctx->sca_records;
+    run.max_sweeps = sweeps_cap(ctx);
+    run.any_sweeps = ctx->sca_any_sweeps;
+    run.sweep = ctx->sweep;
+    run.times = ctx->times.data() + ctx->next_time;
+    run.n_times = ctx->times.size() - ctx->next_time;
+    uint32_t launches = 0;
+    const cudaError_t e = launch_sca(domain_desc(ctx, step), ctx->sca, run, ctx->stream, &launches);
+    ctx->halo_half = run.half;
+    ctx->launches += launches;
+    if (e != cudaSuccess) return cuda_fail(ctx, e, "sweep kernel launch");
+    advance_host(ctx, step);
+    n -= step;
+  }
+  return ASEP_OK;
+}
+
+// SCA: a graph of `windows` (even) tile launches of `len` sweeps each, with
+// their records and the clock moved past them.  It runs at whatever sweep the
+// device clock says, so it can be launched again and again.  `half`: the half
+// of the edge buffer that it begins and ends with.  Captured on a stream of its
+// own, in relaxed mode: other captures go on.
+cudaError_t sca_graph(asep_ctx* ctx, uint32_t windows, uint32_t len, bool records, uint32_t half,
+                      cudaGraphExec_t* exec, uint32_t* launches) {
+  cudaError_t e;
+  if (!ctx->cap_stream && (e = cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking)) != cudaSuccess) {
+    ctx->cap_stream = nullptr;
+    return e;
+  }
+  if ((e = cudaStreamBeginCapture(ctx->cap_stream, cudaStreamCaptureModeRelaxed)) != cudaSuccess) return e;
+  ScaRun run;
+  run.replayed = records;
+  run.halo = ctx->d_halo;
+  run.half = half;
+  run.parts = ctx->d_sca_parts;
+  uint32_t any = 0;
+  run.max_records = records ? sca_max_records(ctx->times.data() + ctx->next_time, ctx->times.size() - ctx->next_time,
+                                              ctx->S, ctx->sca.tiles, ctx->planes, &any) : 0u;
+  run.max_sweeps = run.any_sweeps = len;
+  run.sweep = ctx->sweep;
+  run.times = nullptr;
+  run.n_times = 0;
+  const cudaError_t launched = launch_sca(domain_desc(ctx, windows * len), ctx->sca, run, ctx->cap_stream, launches);
+  cudaGraph_t graph = nullptr;
+  e = cudaStreamEndCapture(ctx->cap_stream, &graph);
+  if (launched != cudaSuccess) e = launched;
+  if (e == cudaSuccess) e = cudaGraphInstantiate(exec, graph, 0);
+  if (graph) cudaGraphDestroy(graph);
+  return e;
+}
+
+// Launches a call of the SCA may put on the stream one by one.  A stream's
+// queue takes some 1024, and a call that has more to enqueue returns only when
+// nearly done: 2^20 sweeps of eight rings of 4096 held the host for 309 of
+// their 353 ms.  Longer calls go as graphs (one place in the queue each, 2 us a
+// launch; 0.5 ms to make one of 256 launches, 5 ms one of 2048), after the
+// remainder, which runs while the graph is made.
+constexpr uint32_t kScaGraph = 256, kScaGraphMost = 2048;
+
+// Whether the next n sweeps may hold sample times (those of replays are later ones than the host knows).
+bool sca_has_records(const asep_ctx* ctx, uint64_t n) {
+  return ctx->next_time < ctx->times.size() && (ctx->replayed || ctx->times[ctx->next_time] <= ctx->sweep + n);
+}
+
+// `times` graphs of `windows` tile launches of `len` sweeps.
+int sca_graphs(asep_ctx* ctx, uint64_t times, uint32_t windows, uint32_t len) {
+  if (!times) return ASEP_OK;
+  const uint64_t each = static_cast<uint64_t>(windows) * len;
+  const bool records = sca_has_records(ctx, times * each);
+  cudaError_t e = cudaSuccess;
+  if (ctx->sca.tiles > 1 && (ctx->replayed || ctx->halo_half == kScaNoHalo)) {
+    if ((e = launch_sca_halo(domain_desc(ctx, 0), ctx->sca, ctx->d_halo, ctx->stream)) != cudaSuccess)
+      return cuda_fail(ctx, e, "edge units");
+    ++ctx->launches;
+    ctx->halo_half = 0;
+  }
+  const uint32_t half = ctx->sca.tiles > 1 ? ctx->halo_half : 0u;
+  cudaGraphExec_t exec = nullptr;
+  uint32_t launches = 0;
+  cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  e = sca_graph(ctx, windows, len, records, half, &exec, &launches);
+  (void)cudaThreadExchangeStreamCaptureMode(&mode);
+  if (e != cudaSuccess) {  // no memory for a graph, say: one by one
+    (void)cudaGetLastError();
+    return sca_direct(ctx, times * each, false);
+  }
+  for (uint64_t k = 0; k < times && e == cudaSuccess; ++k) {
+    if ((e = cudaGraphLaunch(exec, ctx->stream)) != cudaSuccess) break;
+    ctx->launches += launches;
+    advance_host(ctx, each);
+  }
+  cudaGraphExecDestroy(exec);  // one in flight is freed when it is done
+  if (e != cudaSuccess) {
+    ctx->halo_half = kScaNoHalo;
+    return cuda_fail(ctx, e, "graph launch");
+  }
+  return ASEP_OK;
+}
+
+int sweep_sca(asep_ctx* ctx, uint64_t n) {
+  if (is_capturing(ctx->stream)) {
+    ctx->replayed = true;
+    return sca_direct(ctx, n, true);
+  }
+  // Sweeps of a graph's tile launches: with records, as many as the buffer has room for wherever they begin.  (Where
+  // that is far fewer -- from some 10^5 tiles on, dense records -- launches that end where a record does not fit are
+  // the faster ones, and each is long.)
+  const uint32_t full = std::min(sweeps_cap(ctx), kScaTileSweeps);
+  const uint32_t len = sca_has_records(ctx, n) ? std::min(full, ctx->sca_any_sweeps) : full;
+  const uint64_t windows = 2 * len >= full ? n / len : 0;
+  const uint64_t most = windows / kScaGraphMost >= 4 ? windows / kScaGraphMost : 0;
+  const uint64_t some = windows > kScaGraph ? (windows - most * kScaGraphMost) / kScaGraph : 0;
+  const uint64_t graphs = (most * kScaGraphMost + some * kScaGraph) * len;
+  int rc = sca_direct(ctx, n - graphs, false);
+  if (rc == ASEP_OK) rc = sca_graphs(ctx, some, kScaGraph, len);
+  if (rc == ASEP_OK) rc = sca_graphs(ctx, most, kScaGraphMost, len);
+  return rc;
+}
+
 int set_clock(asep_ctx* ctx, uint64_t sweep, uint32_t next_time) {
   const cudaError_t e = launch_set_clock(ctx->d_clock, sweep, next_time, ctx->stream);
   if (e != cudaSuccess) return cuda_fail(ctx, e, "set clock");
@@ -962,13 +1094,12 @@ int asep_create(const asep_params* params, asep_ctx** out) {
 int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
   if (!ctx) return ASEP_ERR_INVALID;
   if (ctx->sweep + n_mcs >= (1ull << 40)) return fail(ctx, ASEP_ERR_INVALID, "sweep index would exceed 2^40");
+  if (ctx->p.schedule == ASEP_SCHED_SCA) return sweep_sca(ctx, n_mcs);
   uint64_t done = 0;
   while (done < n_mcs) {
     uint64_t n = n_mcs - done;
-    uint32_t sweep_launches = 0;  // SCA: counted by the launch, with the clock's
     const uint32_t cap = sweeps_cap(ctx);
-    if (ctx->p.schedule == ASEP_SCHED_SCA) n = std::min<uint64_t>(n, 1u << 20);  // split into launches there
-    else if (n > cap) n = cap;
+    if (n > cap) n = cap;
     cudaError_t e;
     if (ctx->p.schedule == ASEP_SCHED_DOMAIN && ctx->cluster == kStreamTier) {
       // one sweep per step: both phases, lane changes, the record, the clock
@@ -981,22 +1112,6 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
       }
     } else if (ctx->p.schedule == ASEP_SCHED_DOMAIN && ctx->cluster > 1) {
       e = launch_cluster(domain_desc(ctx, static_cast<uint32_t>(n)), ctx->threads, ctx->smem, ctx->stream);
-    } else if (ctx->p.schedule == ASEP_SCHED_SCA) {
-      const bool capturing = is_capturing(ctx->stream);
-      ctx->replayed = ctx->replayed || capturing;
-      ScaRun run;
-      run.replayed = capturing || (ctx->replayed && ctx->next_time < ctx->times.size());
-      run.halo = ctx->d_halo;
-      run.half = ctx->replayed ? kScaNoHalo : ctx->halo_half;  // replays move the lattice on without the host
-      run.parts = ctx->d_sca_parts;
-      run.max_records = ctx->sca_records;
-      run.max_sweeps = cap;
-      run.any_sweeps = ctx->sca_any_sweeps;
-      run.sweep = ctx->sweep;
-      run.times = ctx->times.data() + ctx->next_time;
-      run.n_times = ctx->times.size() - ctx->next_time;
-      e = launch_sca(domain_desc(ctx, static_cast<uint32_t>(n)), ctx->sca, run, ctx->stream, &sweep_launches);
-      ctx->halo_half = run.half;
     } else if (ctx->p.schedule == ASEP_SCHED_DOMAIN && ctx->balance && ctx->cluster == 1 && n > ctx->balance) {
       BalanceLaunch b;
       b.chunk = ctx->balance;
@@ -1030,16 +1145,15 @@ int asep_sweep(asep_ctx* ctx, uint64_t n_mcs) {
       e = launch_serial_plan(a, ctx->p.model, ctx->p.dis_kind, ctx->cluster, ctx->stream);
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "sweep kernel launch");
-    if (ctx->p.schedule != ASEP_SCHED_SCA) {
-      if ((e = launch_advance(ctx->d_clock, ctx->d_times, static_cast<uint32_t>(ctx->times.size()),
-                              static_cast<uint32_t>(n), ctx->stream)) != cudaSuccess)
-        return cuda_fail(ctx, e, "clock advance");
-      // the sweep kernels (streamed domain tier: one per phase, plus the lane
-      // changes with turning sites) and the clock
-      sweep_launches = ctx->cluster != kStreamTier ? 2u
-                       : (ctx->p.dis_kind == ASEP_DIS_TURNING || ctx->p.dis_kind == ASEP_DIS_CROSSING) ? 4u : 3u;
-    }
-    ctx->launches += sweep_launches;
+    if ((e = launch_advance(ctx->d_clock, ctx->d_times, static_cast<uint32_t>(ctx->times.size()),
+                            static_cast<uint32_t>(n), ctx->stream)) != cudaSuccess)
+      return cuda_fail(ctx, e, "clock advance");
+    // the sweep kernels (streamed domain tier: one per phase, plus the lane
+    // changes with turning sites) and the clock
+    uint32_t sweep_launches = 1;
+    if (ctx->cluster == kStreamTier)
+      sweep_launches = (ctx->p.dis_kind == ASEP_DIS_TURNING || ctx->p.dis_kind == ASEP_DIS_CROSSING) ? 3u : 2u;
+    ctx->launches += sweep_launches + 1;
     advance_host(ctx, n);
     done += n;
   }

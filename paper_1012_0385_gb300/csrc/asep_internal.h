@@ -271,6 +271,7 @@ struct ScaPart {
 // has room for its records wherever it begins.
 uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t tiles, uint32_t planes,
                          uint32_t* any_sweeps);
+constexpr uint32_t kScaTileSweeps = 128;  // sweeps a launch: the halo's 256 sites allow no more
 constexpr uint32_t kScaNoHalo = 2;
 // One call's buffers and schedule (host).
 struct ScaRun {
@@ -285,6 +286,8 @@ struct ScaRun {
   size_t n_times;
   bool replayed;           // the launches may run at other sweeps than the host's (captured into a caller's graph)
 };
+// Fills the first half of the buffer from the lattice.
+cudaError_t launch_sca_halo(const DomainLaunch& a, const ScaTiles& tiles, uint32_t* halo, cudaStream_t st);
 // a.n_sweeps sweeps in launches of at most 128, with the records inside them,
 // and the clock moved past them; *launches is advanced.
 cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, ScaRun& run, cudaStream_t st,

@@ -31,8 +31,6 @@
 namespace asep {
 namespace {
 
-constexpr uint32_t kScaTileSweeps = 128;  // sweeps a launch: the halo's 256 sites allow no more
-
 // Two units a thread from here on (one-unit tiles of a launch), for the kinds
 // with a fixed number of planes: the halos cost 3 % instead of 7 %, but a
 // launch then has half the warps, and below some 100 tiles per SM their last
@@ -587,6 +585,14 @@ uint32_t sca_max_records(const uint64_t* times, size_t n, uint32_t S, uint32_t t
   return static_cast<uint32_t>(room);
 }
 
+cudaError_t launch_sca_halo(const DomainLaunch& a, const ScaTiles& tiles, uint32_t* halo, cudaStream_t st) {
+  (void)cudaGetLastError();
+  const size_t n16 = sca_halo_words(tiles, a.geo.S, a.geo.planes) / 8u;
+  const uint32_t blocks = static_cast<uint32_t>(std::min<size_t>((n16 + 255u) / 256u, 152u * 16u));
+  k_sca_halo<<<blocks, 256, 0, st>>>(a.state, halo, a.geo.S, a.geo.planes, a.geo.W, tiles.tiles, tiles.units);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, ScaRun& run, cudaStream_t st,
                        uint32_t* launches) {
   const size_t half = sca_halo_words(tiles, a.geo.S, a.geo.planes) / 2u;
@@ -594,10 +600,7 @@ cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, ScaRun& run
   bool advanced = false;
   (void)cudaGetLastError();
   if (tiles.tiles > 1u && run.half == kScaNoHalo) {
-    const size_t n16 = half / 4u;
-    const uint32_t blocks = static_cast<uint32_t>(std::min<size_t>((n16 + 255u) / 256u, 152u * 16u));
-    k_sca_halo<<<blocks, 256, 0, st>>>(a.state, run.halo, a.geo.S, a.geo.planes, a.geo.W, tiles.tiles, tiles.units);
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_sca_halo(a, tiles, run.halo, st);
     if (e != cudaSuccess) return e;
     ++*launches;
   }
