@@ -12,9 +12,10 @@
 // (lanes 0, 2, ..., 30) and the 16 of word 2g + 1 (lanes 1, 3, ..., 31).
 // Bit k of every lane's u is bit `lane` of random plane k of the group; call k
 // of the stream (tag SCA, ctr3 = 2 * unit + phase) gives plane k of the four
-// groups of a unit (8 words).  The comparison u < t runs most significant bit
-// first over all 32 lanes at once and stops when no lane is undecided or no
-// set bit of any threshold is left (p = 0.75, q = 0.25 need two planes).
+// groups of a unit (8 words).  The comparison u < t runs over all 32 lanes at
+// once, and only over planes down to the lowest set bit of any threshold (p =
+// 0.75, q = 0.25 need two); longer ones end when no lane is undecided
+// (asep_sca.cuh).
 //
 // Layout.  A warp holds a tile of consecutive units of one ring in registers
 // for a whole launch, in the bond-lane form of asep_sca.cuh; the lattice is in
@@ -54,8 +55,8 @@ constexpr uint32_t kScaFewUnits = 4u;
 struct ScaTileLaunch {
   uint32_t tiles, units;  // per ring: tiles, units per tile (the last may hold fewer)
   uint32_t n, offset;     // sweeps of this launch, and before it since the context clock
-  uint32_t n_rec, rec_offset;  // sample times inside this launch, and before it since the clock's cursor
-                               // (kScaReplayed: the device finds them, at most n_rec)
+  uint32_t n_rec, rec_offset;  // sample times inside this launch (at most, if it may run at any sweep), and before
+                               // it since the clock's cursor
   const uint32_t* halo_in;   // [S][tiles][first, last unit][planes][8] (one tile a ring: unused)
   uint32_t* halo_out;
   ScaPart* parts;         // [n_rec + 1][S][tiles][planes] (the last entry: the launch's hops; one tile: unused)
@@ -81,9 +82,10 @@ struct ScaTileLaunch {
 // 173 of 268 instructions a unit and sweep at two planes).  Measured against
 // one CTA per ring with two barriers a sweep, and against one launch per phase
 // with the lattice streamed through HBM, us per sweep: 256 rings of 2^17 at
-// p = 0.75, q = 0.25 1.90 -> 1.65, 201 rings of 391 units with independent
-// classes 13.0 -> 9.0, 128 pairs of lanes of 2^16 with turning sites 6.35 ->
-// 6.5, 2 rings of 2^22 10.3 -> 0.60, 8 rings of 2^28 189 -> 87.
+// p = 0.75, q = 0.25 (hops not counted) 1.90 -> 1.65, 128 pairs of lanes of 2^16
+// with turning sites 6.35 -> 6.6 (units in registers on both sides), 201 rings
+// of 391 units with independent classes 18.7 -> 9.0, 2 rings of 2^22 10.2 -> 0.55,
+// 8 rings of 2^28 191 -> 87 (against the kernels with plain words).
 //
 // Records are taken inside the launch: a tile leaves the sums of its heights
 // relative to its entry height, its height change and its hops so far, and
@@ -96,29 +98,6 @@ struct ScaTileLaunch {
 // the lattice, and a record of it is whole.  It needs neither buffer, which are
 // 128 B of halo a tile and plane and 40 B a record, tile and plane beside 32 B
 // of lattice a unit.
-
-// Sample times of a launch from sweep s0 on: index of the first, and how many.
-// The host knows both, except of a launch that is captured into a graph of the
-// caller's: replays run it at sweeps that only the device clock knows (they
-// then come after the clock's cursor, which k_advance keeps).  All 32 lanes call.
-constexpr uint32_t kScaReplayed = 0xFFFFFFFFu;
-struct ScaTimes {
-  uint32_t first, n;
-};
-__device__ __forceinline__ ScaTimes sca_times(const DomainLaunch& a, const ScaTileLaunch& t, uint64_t s0) {
-  const uint32_t next = a.clock->next_time;
-  if (t.rec_offset != kScaReplayed) return {next + t.rec_offset, t.n_rec};
-  const uint32_t lane = threadIdx.x & 31u;
-  // times are ascending: how many from `from` on are at most `last`, no more than `most`
-  const auto count = [&](uint32_t from, uint64_t last, uint32_t most) {
-    uint32_t n = 0;
-    for (uint32_t c = 32; c == 32u && n < most; n += c)
-      c = __popc(__ballot_sync(0xffffffffu, from + n + lane < a.n_times && a.times[from + n + lane] <= last));
-    return min(n, most);
-  };
-  const uint32_t first = next + count(next, s0, a.n_times);
-  return {first, count(first, s0 + t.n, t.n_rec)};
-}
 
 // The tile's hops since the launch began.
 __device__ __forceinline__ void tile_hops(const ScaCounts& cnt, ScaPart* part) {
@@ -231,6 +210,9 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
 
   // local unit i = lane UPT + j: 0 and n_own + 1 are the halos
   uint32_t* state = a.state + static_cast<size_t>(sample) * NOCC * W;
+  // A launch that may run at any sweep -- captured into a graph -- knows only how many sample times can fall into it.
+  const uint64_t* next_time = a.times + a.clock->next_time + t.rec_offset;
+  const auto more = [&](uint32_t r) { return r < t.n_rec && next_time + r < a.times + a.n_times; };
   const size_t edge0 = static_cast<size_t>(sample) * t.tiles * 2u;  // this ring's entries of the halo buffers
   uint32_t gu[UPT], counted[UPT];
   ScaUnit U[NOCC][UPT];
@@ -244,13 +226,12 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
     if (g >= n_units) g -= n_units;
     gu[j] = g;
     counted[j] = own ? ~0u : 0u;
-    const uint32_t* src = state + 8u * g;
-    size_t pitch = W;
-    if (used && !own && t.tiles > 1u) {  // left halo: the previous tile's last unit; right halo: the next tile's first
-      const uint32_t nb = i == 0u ? (tile == 0u ? t.tiles : tile) - 1u : (tile + 1u == t.tiles ? 0u : tile + 1u);
-      src = t.halo_in + (edge0 + 2u * nb + (i == 0u ? 1u : 0u)) * (NOCC * 8u);
-      pitch = 8;
-    }
+    // left halo: the previous tile's last unit; right halo: the next tile's first
+    const uint32_t nb = i == 0u ? (tile == 0u ? t.tiles : tile) - 1u : (tile + 1u == t.tiles ? 0u : tile + 1u);
+    const uint32_t* edge = t.halo_in + (edge0 + 2u * nb + (i == 0u ? 1u : 0u)) * (NOCC * 8u);
+    const bool from_edges = used && !own && t.tiles > 1u;
+    const uint32_t* src = from_edges ? edge : state + 8u * g;
+    const uint32_t pitch = from_edges ? 8u : W;
 #pragma unroll
     for (uint32_t p = 0; p < NOCC; ++p) {
       uint32_t x[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
@@ -281,8 +262,6 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
   ScaCounts cnt;
   const size_t part_pitch = static_cast<size_t>(a.geo.S) * t.tiles * NOCC;  // entries of one record
   ScaPart* part = t.parts + (static_cast<size_t>(sample) * t.tiles + tile) * NOCC;
-  const ScaTimes rec_times = sca_times(a, t, s0);
-  const uint64_t* next_time = a.times + rec_times.first;
   uint32_t filled = 0, base = 0, recs = 0;
   for (uint32_t done = 0; done < t.n;) {
     if (done == filled) {
@@ -293,7 +272,7 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
       __syncwarp();
     }
     uint32_t stop = filled;
-    if (recs < rec_times.n) stop = static_cast<uint32_t>(min(static_cast<uint64_t>(stop), next_time[recs] - s0));
+    if (more(recs)) stop = static_cast<uint32_t>(min(static_cast<uint64_t>(stop), next_time[recs] - s0));
 #pragma unroll 1
     for (; done < stop; ++done) {
       const uint32_t it = done - base;
@@ -354,13 +333,14 @@ __global__ void __launch_bounds__(32, DIS ? 20 : (MODEL == kTwoLane ? 24 : 28))
                        : sca_turn_pool<1>(U[0][0], U[NOCC - 1][0], Q[0], *turn, gu[0], counted[0], a0, b2,
                                           hd[kmax + 1], a);
     }
-    if (recs < rec_times.n && next_time[recs] == s0 + done) {
-      tile_record<NOCC, UPT>(U, gu, counted, a, sample, s0 + done, rec_times.first + recs, t.tiles == 1u,
-                             part + recs * part_pitch, COUNT, cnt);
+    if (more(recs) && next_time[recs] == s0 + done) {
+      tile_record<NOCC, UPT>(U, gu, counted, a, sample, s0 + done, next_time + recs - a.times, t.tiles == 1u,
+                             part, COUNT, cnt);
+      part += part_pitch;
       ++recs;
     }
   }
-  if (COUNT && t.n_rec && t.tiles > 1u) tile_hops(cnt, part + t.n_rec * part_pitch);
+  if (COUNT && t.n_rec && t.tiles > 1u) tile_hops(cnt, part + (t.n_rec - recs) * part_pitch);
 
 #pragma unroll
   for (uint32_t j = 0; j < UPT; ++j) {
@@ -401,9 +381,8 @@ __device__ __forceinline__ void sca_records(const DomainLaunch& a, const ScaTile
   const uint32_t S = a.geo.S, planes = a.geo.planes, n_units = a.geo.W / 8u;
   if (item >= static_cast<uint64_t>(t.n_rec) * S) return;  // whole warps
   const uint32_t r = static_cast<uint32_t>(item / S), sample = static_cast<uint32_t>(item - static_cast<uint64_t>(r) * S);
-  const ScaTimes times = sca_times(a, t, a.clock->sweep + t.offset);
-  if (r >= times.n) return;  // whole warps
-  const size_t slot = static_cast<size_t>(times.first) + r;
+  const size_t slot = static_cast<size_t>(a.clock->next_time) + t.rec_offset + r;
+  if (slot >= a.n_times || a.times[slot] > a.clock->sweep + t.offset + t.n) return;  // whole warps
   const ScaPart* mine = t.parts + (static_cast<size_t>(r) * S + sample) * t.tiles * planes;
   const ScaPart* after = t.parts + (static_cast<size_t>(t.n_rec) * S + sample) * t.tiles * planes;
   long long hops[4] = {0, 0, 0, 0};
@@ -597,7 +576,6 @@ cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, ScaRun& run
                        uint32_t* launches) {
   const size_t half = sca_halo_words(tiles, a.geo.S, a.geo.planes) / 2u;
   uint32_t rec = 0;
-  bool advanced = false;
   (void)cudaGetLastError();
   if (tiles.tiles > 1u && run.half == kScaNoHalo) {
     const cudaError_t e = launch_sca_halo(a, tiles, run.halo, st);
@@ -612,8 +590,9 @@ cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, ScaRun& run
     t.units = tiles.units;
     t.n = std::min({kScaTileSweeps, run.max_sweeps, a.n_sweeps - done});
     if (run.replayed) t.n = std::min(t.n, run.any_sweeps);
-    t.offset = done;
-    t.rec_offset = run.replayed ? kScaReplayed : rec;
+    // a launch that may run at any sweep finds its records from the clock, which then moves with every launch
+    t.offset = run.replayed ? 0u : done;
+    t.rec_offset = run.replayed ? 0u : rec;
     t.n_rec = run.replayed ? std::min(t.n, run.max_records) : 0u;
     while (!run.replayed && rec + t.n_rec < run.n_times && run.times[rec + t.n_rec] - run.sweep <= done + t.n) {
       if (t.n_rec == run.max_records) {  // the launch ends before the first record it has no room for
@@ -628,21 +607,20 @@ cudaError_t launch_sca(const DomainLaunch& a, const ScaTiles& tiles, ScaRun& run
     cudaError_t e = launch_tiles(a, t, tiles.upt, st);
     if (e != cudaSuccess) return e;
     ++*launches;
+    uint32_t advance = done + t.n < a.n_sweeps ? 0u : a.n_sweeps;
+    if (run.replayed) advance = t.n;
     if (t.n_rec && tiles.tiles > 1u) {
       const uint64_t items = static_cast<uint64_t>(t.n_rec) * a.geo.S;
-      advanced = done + t.n == a.n_sweeps;
-      k_sca_records<<<static_cast<uint32_t>((items + 3u) / 4u), 128, 0, st>>>(a, t, advanced ? a.n_sweeps : 0u);
+      k_sca_records<<<static_cast<uint32_t>((items + 3u) / 4u), 128, 0, st>>>(a, t, advance);
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
+      ++*launches;
+    } else if (advance) {
+      if ((e = launch_advance(a.clock, a.times, a.n_times, advance, st)) != cudaSuccess) return e;
       ++*launches;
     }
     half_now ^= 1u;
     rec += t.n_rec;
     done += t.n;
-  }
-  if (!advanced) {
-    const cudaError_t e = launch_advance(a.clock, a.times, a.n_times, a.n_sweeps, st);
-    if (e != cudaSuccess) return e;
-    ++*launches;
   }
   run.half = half_now;
   return cudaSuccess;
