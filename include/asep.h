@@ -224,14 +224,16 @@ int asep_plan(const asep_params* params, asep_info* info);
  * be captured into a CUDA graph of the caller's: replays continue from the
  * device's sweep count, but what the host reports (asep_info, how many records
  * the tables hold) counts calls, not replays, until asep_load_state or
- * asep_reset sets both. */
+ * asep_reset sets both; streamed domain plans also place their records by the
+ * host's count. */
 int asep_sweep(asep_ctx* ctx, uint64_t n_mcs);
 
 /* Copy the heights recorded so far.  Entry e = (time index, sample, plane),
  * layout [n_recorded][S][planes]: sum_h[e] = sum_i h_i with
  * h_i = sum_{j<=i} (2 n_j - 1); sum_h2[2e], sum_h2[2e+1] = low and high words
  * of the unsigned 128-bit sum_i h_i^2; w2[e] = W^2 of Eq. (W) (paper sec.
- * 2.1) = (L sum h^2 - (sum h)^2) / L^2, evaluated exactly then rounded.  Any
+ * 2.1) = (L sum h^2 - (sum h)^2) / L^2, the quotient of exact integers to
+ * within one unit in the last place.  Any
  * output pointer may be NULL.  n_entries must be >= n_recorded*S*planes.
  * Synchronises the context stream. */
 int asep_width(asep_ctx* ctx, int64_t* sum_h, uint64_t* sum_h2, double* w2, size_t n_entries);

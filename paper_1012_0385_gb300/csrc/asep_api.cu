@@ -288,13 +288,6 @@ size_t sca_parts_bytes(const asep_ctx* ctx) {
   return (ctx->sca_records + static_cast<size_t>(1)) * ctx->S * ctx->sca.tiles * ctx->planes * sizeof(ScaPart);
 }
 
-// Launch plan.  Resident: columns = super-domains, one thread per column, a
-// whole sample (or several small ones) per CTA.  Cluster tier: each sample
-// spread over 2..16 CTAs of a thread-block cluster, for samples one CTA
-// cannot hold -- or, on request, to spread few large samples over more SMs.
-// force_cluster: 0 = choose, 1 = resident only, n > 1 = exactly n CTAs per
-// sample.  force_spc: samples per CTA for the resident plan (0 = choose).
-// The plan changes only the launch shape, never the results.
 int sm_count() {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -385,6 +378,15 @@ void plan_spread(asep_ctx* ctx, bool automatic) {
 // Automatic tile width of the streamed tier, in columns (one thread each).
 constexpr uint32_t kStreamTileColumns = 128;
 
+// Launch plan of the domain schedule.  Resident: columns = super-domains, one
+// thread per column, a whole sample (or several small ones) per CTA.  Cluster
+// tier: each sample spread over 2..16 CTAs of a thread-block cluster, for
+// samples one CTA cannot hold or, few of them, to use more SMs (spreads).
+// Streamed: tiles of columns, the lattice in global memory.
+// force_cluster: 0 = choose, 1 = resident only, kStreamTier = streamed, other n
+// > 1 = exactly n CTAs per sample.  force_spc: samples per CTA for the resident
+// plan, columns per tile for the streamed one (0 = choose).
+// The plan changes only the launch shape, never the results.
 int plan_domain(asep_ctx* ctx, uint32_t force_cluster, uint32_t force_spc) {
   const uint32_t D = ctx->D;
   ctx->R2 = 2 * D / 32;
@@ -716,12 +718,13 @@ cudaError_t sca_graph(asep_ctx* ctx, uint32_t windows, uint32_t len, bool record
   return e;
 }
 
-// Launches a call of the SCA may put on the stream one by one.  A stream's
-// queue takes some 1024, and a call that has more to enqueue returns only when
-// nearly done: 2^20 sweeps of eight rings of 4096 held the host for 309 of
-// their 353 ms.  Longer calls go as graphs (one place in the queue each, 2 us a
-// launch; 0.5 ms to make one of 256 launches, 5 ms one of 2048), after the
-// remainder, which runs while the graph is made.
+// Launches of tiles that a call of the SCA may put on the stream one by one, and
+// those of a graph (the larger for long calls).  A stream's queue takes some
+// 1024, and a call that has more to enqueue returns only when nearly done: 2^20
+// sweeps of eight rings of 4096 held the host for 309 of their 353 ms.  Longer
+// calls go as graphs (one place in the queue each, 2 us a launch; 0.5 ms to make
+// one of 256 launches, 5 ms one of 2048), after the remainder, which runs while
+// the graph is made.
 constexpr uint32_t kScaGraph = 256, kScaGraphMost = 2048;
 
 // Whether the next n sweeps may hold sample times (those of replays are later ones than the host knows).
@@ -1243,8 +1246,9 @@ int asep_width(asep_ctx* ctx, int64_t* sum_h, uint64_t* sum_h2, double* w2, size
       const unsigned __int128 s2 = (static_cast<unsigned __int128>(sh2[2 * i + 1]) << 64) | sh2[2 * i];
       const __int128 s1 = sh[i];
       const unsigned __int128 num = ctx->L * s2 - static_cast<unsigned __int128>(s1 * s1);  // >= 0, < 2^110
-      // num / L^2 with one rounding: split into integer quotient and remainder, which 64 bits hold for all but the
-      // longest rings (a 128-bit division is a library call: 0.6 ms of a call on 26 000 entries)
+      // num / L^2 from its integer quotient and remainder, both exact: within one unit in the last place (the
+      // remainder's share of one rounds before the sum does).  64 bits hold them for all but the longest rings (a
+      // 128-bit division is a library call: 0.6 ms of a call on 26 000 entries)
       if (((num | L2) >> 64) == 0) {
         const uint64_t n64 = static_cast<uint64_t>(num), d64 = static_cast<uint64_t>(L2);
         w2[i] = static_cast<double>(n64 / d64) + static_cast<double>(n64 % d64) / static_cast<double>(d64);

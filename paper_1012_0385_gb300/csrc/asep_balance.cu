@@ -4,10 +4,9 @@
 // CTAs each leaves some SMs with one group and others with two for the whole
 // launch (256 samples on 152 SMs: 104 SMs with two, 48 with one).  The SMs
 // with two bound the launch, while the others run half loaded.  Here the
-// launch's sweeps are cut into chunks and a persistent grid --
-// ceil(groups / SMs) CTAs per SM, so one slot per SM beyond the groups'
-// share floats -- takes (sample group, chunk) items from a queue in
-// chunk-major order.  A CTA runs chunk k of a group once chunk k - 1 of
+// launch's sweeps are cut into chunks and a persistent grid -- slots for some
+// 17 warps per SM and no more than the groups need, ceil(groups / SMs) -- takes
+// (sample group, chunk) items from a queue in chunk-major order.  A CTA runs chunk k of a group once chunk k - 1 of
 // that group has published its lattice, so groups move between SMs between
 // chunks, and an SM whose second slot is free takes the next item.  Each
 // group's sweeps still run in order from the lattice its previous chunk left

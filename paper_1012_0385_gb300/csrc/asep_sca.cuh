@@ -283,7 +283,7 @@ __device__ __forceinline__ void decide_lane(const uint32_t (&cand)[4], uint32_t 
 }
 
 struct ScaCounts {
-  uint32_t c[4] = {0u, 0u, 0u, 0u};  // at most 512 a sweep and unit, 2^20 sweeps a launch
+  uint32_t c[4] = {0u, 0u, 0u, 0u};  // at most 512 a sweep and unit, 128 sweeps a launch
 };
 
 // One phase of one unit of lane P (ring: P = 0), given the phase's first
