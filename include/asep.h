@@ -220,7 +220,9 @@ int asep_plan(const asep_params* params, asep_info* info);
  * recording heights after every sweep count listed in sample_times.
  * Asynchronous: returns once the work is enqueued (the SCA puts a call of more
  * than 256 launches, 32768 sweeps, on the stream as CUDA graphs, so that it
- * fits the stream's queue; making them takes the host 0.5 to 6 ms).  A call may
+ * fits the stream's queue; making them takes the host 0.5 to 6 ms and the driver
+ * a few MB of device memory until they are done; where that fails the launches
+ * go one by one and the call returns when the queue has taken them).  A call may
  * be captured into a CUDA graph of the caller's: replays continue from the
  * device's sweep count, but what the host reports (asep_info, how many records
  * the tables hold) counts calls, not replays, until asep_load_state or
